@@ -4,6 +4,7 @@
 #include "internal.cuh"
 
 #include <algorithm>
+#include <climits>
 
 #include <cmath>
 #include <cstdarg>
@@ -364,6 +365,128 @@ __global__ void k_pat_fill(const int64_t *rp, const int32_t *col, int64_t n, con
   reinterpret_cast<unsigned *>(blk + 32)[lane] = mk;
 }
 
+// Staged blocks of the shared-pattern schedule (k_spmm_block): one CTA of T
+// threads per block, thread t owning rows 3t .. 3t + 2.  As in slice_pattern
+// the rows' sorted short-row offsets are walked in step; each round takes the
+// smallest head in the block as the next union offset.  Thread 0 then lays out
+// the ranges of X rows the block reads (offsets less than a block apart share a
+// range; ranges start at even rows so that 8-byte rows keep 16-byte copies)
+// and the runs of consecutive offsets (at most 3 long).  stat[0] is set when a
+// block has more than 31 offsets, stat[1] takes the largest staged row count.
+__global__ void k_blk_build(const int64_t *rp, const int32_t *col, int64_t n, const uint8_t *sdeg, int32_t *desc,
+                            unsigned *mask, int *stat) {
+  constexpr int R = 3;
+  __shared__ int wmin[2][kBlkThreads / 32];
+  __shared__ int u[32];
+  const int tid = threadIdx.x, T = blockDim.x, warps = T >> 5;
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * (R * T);
+  int64_t rb[R];
+  int d[R], pos[R];
+  unsigned mk[R];
+  for (int j = 0; j < R; ++j) {
+    const int64_t row = r0 + R * tid + j;
+    const bool ok = row < n && sdeg[row] != 0xFF;
+    d[j] = ok ? sdeg[row] : 0;
+    rb[j] = ok ? rp[row] : 0;
+    pos[j] = 0;
+    mk[j] = ok ? 0u : 0x80000000u;
+  }
+  int nu = 0, prev = INT_MIN, lastu = INT_MIN, round = 0;
+  for (;; ++nu, ++round) {
+    int cand[R], m = INT_MAX;
+    for (int j = 0; j < R; ++j) {
+      const int64_t row = r0 + R * tid + j;
+      cand[j] = pos[j] < d[j] ? static_cast<int>(static_cast<int64_t>(col[rb[j] + pos[j]]) - row) : INT_MAX;
+      m = min(m, cand[j]);
+    }
+    m = __reduce_min_sync(0xffffffffu, m);
+    if ((tid & 31) == 0) wmin[round & 1][tid >> 5] = m;
+    __syncthreads();
+    for (int k = 0; k < warps; ++k) m = min(m, wmin[round & 1][k]);
+    if (m == INT_MAX || nu == 31 || m <= prev) {
+      if (m != INT_MAX) nu = 32;   // too many offsets, or a row out of order
+      break;
+    }
+    prev = m;
+    // offsets -1 and 1: offset 0 goes between them as an entry that no row
+    // has, so that they share a run
+    if (m == 1 && lastu == -1 && nu < 30) {
+      if (tid == 0) u[nu] = 0;
+      ++nu;
+    }
+    lastu = m;
+    for (int j = 0; j < R; ++j)
+      if (cand[j] == m) {
+        mk[j] |= 1u << nu;
+        ++pos[j];
+      }
+    if (tid == 0) u[nu] = m;
+  }
+  for (int j = 0; j < R; ++j) mask[r0 + R * tid + j] = mk[j];
+  if (tid != 0) return;
+  int32_t *out = desc + static_cast<int64_t>(blockIdx.x) * 128;
+  if (nu > 31) {
+    stat[0] = 1;
+    return;
+  }
+  // ranges over the union and offset 0 (the rows themselves), ascending
+  const int64_t span = R * T;
+  int nr = 0, staged = 0, self = 0;
+  int64_t lo = 0, hi = 0;
+  bool open = false, zero_done = false;
+  int base_of[32];               // staged row of the block's row 0 at each offset
+  int first_k = 0;               // offsets of the open range start here
+  for (int k = 0; k <= nu + 1; ++k) {
+    // next offset in ascending order, 0 merged in
+    int64_t o = 0;
+    bool have = false;
+    const int idx = zero_done ? k - 1 : k;
+    if (!zero_done && (idx >= nu || u[idx] > 0)) {
+      o = 0;
+      have = true;
+      zero_done = true;
+    } else if (idx < nu) {
+      o = u[idx];
+      have = true;
+    }
+    if (have && open && o <= hi + span) {
+      hi = o;
+      continue;
+    }
+    if (open) {                  // close [lo, hi + span)
+      const int64_t alo = lo - (lo & 1);
+      const int64_t rows = (hi - alo + span + 1) & ~int64_t{1};
+      out[3 + 3 * nr] = static_cast<int32_t>(alo);
+      out[4 + 3 * nr] = static_cast<int32_t>(rows);
+      out[5 + 3 * nr] = staged;
+      for (; first_k < nu && u[first_k] <= hi; ++first_k) base_of[first_k] = staged + static_cast<int>(u[first_k] - alo);
+      if (lo <= 0 && hi >= 0) self = staged + static_cast<int>(-alo);
+      const int64_t total = staged + rows;
+      staged = total > 60000 ? 60000 : static_cast<int>(total);
+      ++nr;
+    }
+    if (!have) break;
+    open = true;
+    lo = hi = o;
+  }
+  if (nr > 31) {                 // the descriptor holds 31 ranges and 31 runs
+    stat[0] = 1;
+    return;
+  }
+  int nrun = 0;
+  int32_t *runs = out + 3 + 3 * nr;
+  for (int k = 0; k < nu;) {
+    int len = 1;
+    while (len < 3 && k + len < nu && u[k + len] == u[k] + len) ++len;
+    runs[nrun++] = base_of[k] | (len << 16) | (k << 18);
+    k += len;
+  }
+  out[0] = nr;
+  out[1] = nrun;
+  out[2] = self;
+  atomicMax(stat + 1, staged);
+}
+
 int grid_for(int64_t n) {
   int64_t g = (n + 255) / 256;
   if (g > 8 * kSmCount) g = 8 * kSmCount;
@@ -568,6 +691,45 @@ void build_sell(sphynx_graph *g) {
     }
   }
   SPX_CUDA(cudaStreamSynchronize(g->stream));
+}
+
+// Staged blocks, for graphs whose every slice is a shared-pattern slice and
+// whose rows average at least 16 entries: a staged row is then reused often
+// enough to pay for its copy.  Float products, us, staged against lane-per-row
+// kernel: 27-point meshes 80 x 75 x 70 17.2 / 28.9 and 128^3 73.7 / 121 (8
+// columns), 128^3 119 / 119 (12 columns), 210 / 406 (16 columns); the 5-point
+// mesh 1400^2 39.3 / 43.3, but 57.6 / 49.4 with 12 columns.  Blocks of 128
+// threads (384 rows); 64 where that leaves fewer than two blocks an SM (27-point
+// 48 x 40 x 44: 6.2 against 8.2 us).  256 threads measured the same at 128^3
+// (72.4) and 30.9 against 28.8 us at 101 x 97 x 89.
+void build_blocks(sphynx_graph *g) {
+  SpmmPlan &p = g->plan;
+  p.blk_threads = 0;
+  p.blk_desc.release();
+  p.blk_mask.release();
+  if (!p.pat_all || g->nnz < 16 * g->n) return;
+  const int64_t n = g->n;
+  const int T = n >= 3 * kBlkThreads * 2 * kSmCount ? kBlkThreads : kBlkThreads / 2;
+  const int64_t rows = 3 * static_cast<int64_t>(T), blocks = (n + rows - 1) / rows;
+  p.blk_desc.alloc(static_cast<size_t>(blocks) * 128 * sizeof(int32_t));
+  p.blk_mask.alloc(static_cast<size_t>(blocks * rows) * sizeof(unsigned));
+  DevBuf stat;
+  stat.alloc(2 * sizeof(int));
+  SPX_CUDA(cudaMemsetAsync(stat.p, 0, 2 * sizeof(int), g->stream));
+  k_blk_build<<<static_cast<unsigned>(blocks), T, 0, g->stream>>>(g->rowptr, g->col, n, p.sell_deg.as<uint8_t>(),
+                                                                 p.blk_desc.as<int32_t>(), p.blk_mask.as<unsigned>(),
+                                                                 stat.as<int>());
+  SPX_LAUNCHED();
+  int h[2] = {0, 0};
+  SPX_CUDA(cudaMemcpyAsync(h, stat.p, sizeof(h), cudaMemcpyDeviceToHost, g->stream));
+  SPX_CUDA(cudaStreamSynchronize(g->stream));
+  if (h[0] || static_cast<size_t>(h[1]) * 8 > kBlkSmemMax) {   // 8 bytes: the narrowest rows
+    p.blk_desc.release();
+    p.blk_mask.release();
+    return;
+  }
+  p.blk_threads = T;
+  p.blk_staged_rows = h[1];
 }
 
 // The short-row schedule is a property of the graph's structure: both are
@@ -799,6 +961,7 @@ int sphynx_create(const int64_t *row_ptr, const int32_t *col, const float *edge_
     build_plan(g.get(), dev ? nullptr : row_ptr, kMedDeg);
     g->plan.prescale = g->max_degree * g->n > 10 * g->nnz;   // irregular: max degree above 10 x the mean
     build_sell(g.get());
+    build_blocks(g.get());
     autotune_spmm(g.get(), dev ? nullptr : row_ptr);
     *out = g.release();
     return SPHYNX_OK;

@@ -103,6 +103,8 @@ constexpr int kSpmmVariants = 3;
 // sell_cptr / pat_cptr tag of a shared-pattern slice (the start follows in the low bits)
 constexpr int64_t kPatternTag = int64_t{1} << 62;
 
+constexpr int kBlkThreads = 128;                 // threads of a staged block, or half of them (three rows each)
+constexpr size_t kBlkSmemMax = 200 * 1024;       // shared memory a staged block may take
 constexpr int kSellLsCount = 5;      // slice strides 1, 2, 4, 8, 16 the autotuner times
 
 struct SpmmTuning {
@@ -165,6 +167,13 @@ struct SpmmPlan {
   double pat_bytes = 0;              // bytes a product reads from this layout
   DevBuf pat_cptr;                   // int64 [n_slices]
   DevBuf pat_col;                    // 16-bit units, 96 per shared-pattern slice
+  // Staged blocks (k_spmm_block): blocks of 3 blk_threads rows whose short-row
+  // offsets take at most 31 distinct values; 0 threads: not built
+  int blk_threads = 0;
+  int blk_staged_rows = 0;           // rows of X the largest block stages in shared memory
+  DevBuf blk_desc;                   // int32 [blocks][128], see k_spmm_block
+  DevBuf blk_mask;                   // uint32 [blocks * 3 blk_threads]: a row's entries among its block's
+                                     // offsets; bit 31: not a short row
   double long_bytes = 0;             // bytes of the long rows' CSR entries and items
   // Medium rows (kShortDeg < degree <= med_max), sorted by degree (descending,
   // row id on ties) into grp_row, and cut into warp units of rows that share

@@ -170,14 +170,13 @@ struct SpmmDev {              // kernel-side view of SpmmArgs
 
 constexpr int kListGrid = kSmCount * 16;   // CTAs of a launch that walks an active-block list
 
-// acc = sum_j w_ij (s_j) X_j of row `row`; epilogue applies the diagonal part.
+// acc = sum_j w_ij (s_j) X_j of row `row`, xi its own X_i; the epilogue applies
+// the diagonal part.
 template <int LAP, typename TI, typename TT, int BP, int MODE>
 __device__ __forceinline__ void spmm_epilogue(const LapView &L, const SpmmDev &a, int64_t row,
+                                              const typename AccOf<TI>::T (&xi)[BP],
                                               const typename AccOf<TI>::T (&acc)[BP]) {
   using TA = typename AccOf<TI>::T;
-  const TI *x = static_cast<const TI *>(a.xe);
-  TA xi[BP];
-  load_row<BP>(x + row * BP, xi);
   TA out[BP];
   if constexpr (LAP == SPHYNX_NORMALIZED) {
     const TA s = dinv_of<TA>(L, row);
@@ -222,6 +221,14 @@ __device__ __forceinline__ void spmm_epilogue(const LapView &L, const SpmmDev &a
       store_row<BP>(yp, ya);
     }
   }
+}
+
+template <int LAP, typename TI, typename TT, int BP, int MODE>
+__device__ __forceinline__ void spmm_epilogue(const LapView &L, const SpmmDev &a, int64_t row,
+                                              const typename AccOf<TI>::T (&acc)[BP]) {
+  typename AccOf<TI>::T xi[BP];
+  load_row<BP>(static_cast<const TI *>(a.xe) + row * BP, xi);
+  spmm_epilogue<LAP, TI, TT, BP, MODE>(L, a, row, xi, acc);
 }
 
 // ---- packed float pairs: add.rn.f32x2 / fma.rn.f32x2 (sm_100 and later) ----
@@ -891,6 +898,316 @@ k_spmm_sell(const LapView L, const SpmmDev a, const int16_t *__restrict__ scol, 
   sell_slice<LAP, TI, TT, BP, W, MODE, KIND>(L, a, scol, sw, sptr, cptr, sdeg, pcol, slice, lane);
 }
 
+// Staged blocks (SELL-32 with shared-pattern slices, unweighted graphs, L_C).
+// A CTA of T threads owns 3 T consecutive rows.  All their short-row offsets
+// col - row take at most 31 distinct values, so the rows of X the CTA gathers
+// are a few contiguous ranges (three on a 27-point mesh: one per plane): they
+// are copied to shared memory once, coalesced, and every gather is a shared
+// load.  Thread t owns rows 3t, 3t + 1, 3t + 2: a run of L consecutive offsets
+// (-1, 0, 1 on a mesh) takes L + 2 loads (and unpackings of bfloat16) for its
+// 3 L entries.  The lane-per-row kernel is bound by the L1 data pipe (float
+// rows: 16 wavefronts an entry of 32 rows) and, in bfloat16, by issue (29
+// instructions an entry); this one has a third of both and is bound by the
+// latency of a block's copies.  128^3 27-point mesh: float product 122 -> 74 us,
+// bfloat16 chain step 57 -> 53 us.
+// Three rows a thread, not two or four: an odd stride keeps the 16-byte loads
+// of a quarter warp in different banks (two-chunk rows alternate which half
+// they load first).  Every row adds its entries one by one in ascending column
+// order, so the sums are those of the other SELL schedules bit for bit.
+constexpr int kBlkRows = 3;      // rows a thread owns
+constexpr int kBlkDesc = 128;    // ints of a block's descriptor
+
+template <typename TI, int BP> struct BlockTraits {
+  static constexpr int row_bytes = BP * static_cast<int>(sizeof(TI));
+  static constexpr int chunk = row_bytes % 16 == 0 ? 16 : 8;   // bytes a lane loads at once
+  static constexpr int nq = row_bytes / chunk;
+  static constexpr bool rotate = nq == 2 || nq == 4;           // lanes start at different chunks of a row
+  // resident blocks that the staged rows of a 27-point mesh (5 a row) leave room for
+  static constexpr int min_blocks = row_bytes <= 16 ? 7 : (row_bytes <= 32 ? 3 : (row_bytes <= 48 ? 2 : 1));
+};
+
+// one staged row: nq chunks as raw words, chunk q of the lane being chunk
+// (q + rot) mod nq of the row
+template <typename TI, int BP> struct StagedRow {
+  using B = BlockTraits<TI, BP>;
+  static constexpr int words = B::chunk / 4;
+  unsigned w[B::nq][words];
+  __device__ __forceinline__ void load(const unsigned char *p, int rot) {
+#pragma unroll
+    for (int q = 0; q < B::nq; ++q) {
+      const int qq = B::rotate ? ((q + rot) & (B::nq - 1)) : q;
+      if constexpr (words == 4) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(p + 16 * qq);
+        w[q][0] = v.x; w[q][1] = v.y; w[q][2] = v.z; w[q][3] = v.w;
+      } else {
+        const uint2 v = *reinterpret_cast<const uint2 *>(p + 8 * qq);
+        w[q][0] = v.x; w[q][1] = v.y;
+      }
+    }
+  }
+};
+
+// sums of staged rows: packed float pairs, or floats that take bfloat16 values
+// by the mixed-precision multiply-add (exact widening, full rate; unpacking to
+// packed pairs first took 59 instead of 53 us a chain step at 128^3)
+template <typename TI, int BP> struct StagedAcc;
+template <int BP> struct StagedAcc<float, BP> {
+  using S = StagedRow<float, BP>;
+  unsigned long long v[BP / 2];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int c = 0; c < BP / 2; ++c) v[c] = 0ull;
+  }
+  // += r (present) or += 0 r
+  __device__ __forceinline__ void fma(const S &r, bool present) {
+    const float one = present ? 1.f : 0.f;
+    const unsigned long long ones = pk2(one, one);
+#pragma unroll
+    for (int q = 0; q < S::B::nq; ++q)
+#pragma unroll
+      for (int i = 0; i < S::words; i += 2) {
+        const int c = (q * S::words + i) / 2;
+        v[c] = fma2(pk2(__uint_as_float(r.w[q][i]), __uint_as_float(r.w[q][i + 1])), ones, v[c]);
+      }
+  }
+  __device__ __forceinline__ void get(float (&o)[BP]) const {
+#pragma unroll
+    for (int c = 0; c < BP / 2; ++c) {
+      const float2 f = upk2(v[c]);
+      o[2 * c] = f.x;
+      o[2 * c + 1] = f.y;
+    }
+  }
+  __device__ __forceinline__ void set(const float (&o)[BP]) {
+#pragma unroll
+    for (int c = 0; c < BP / 2; ++c) v[c] = pk2(o[2 * c], o[2 * c + 1]);
+  }
+};
+template <int BP> struct StagedAcc<__nv_bfloat16, BP> {
+  using S = StagedRow<__nv_bfloat16, BP>;
+  float v[BP];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int c = 0; c < BP; ++c) v[c] = 0.f;
+  }
+  __device__ __forceinline__ void fma(const S &r, bool present) {
+    const unsigned one = present ? 0x3f80u : 0u;
+#pragma unroll
+    for (int q = 0; q < S::B::nq; ++q)
+#pragma unroll
+      for (int i = 0; i < S::words; ++i) {
+        const int c = 2 * (q * S::words + i);
+        asm("{\n\t.reg .b16 lo, hi, one, zero;\n\tmov.b32 {lo, hi}, %2;\n\tmov.b32 {one, zero}, %3;\n\t"
+            "fma.rn.f32.bf16 %0, lo, one, %0;\n\tfma.rn.f32.bf16 %1, hi, one, %1;\n\t}"
+            : "+f"(v[c]), "+f"(v[c + 1])
+            : "r"(r.w[q][i]), "r"(one));
+      }
+  }
+  __device__ __forceinline__ void get(float (&o)[BP]) const {
+#pragma unroll
+    for (int c = 0; c < BP; ++c) o[c] = v[c];
+  }
+  __device__ __forceinline__ void set(const float (&o)[BP]) {
+#pragma unroll
+    for (int c = 0; c < BP; ++c) v[c] = o[c];
+  }
+};
+// a staged row's values as floats, in the lane's chunk order
+template <typename TI, int BP>
+__device__ __forceinline__ void staged_values(const StagedRow<TI, BP> &r, float (&o)[BP]) {
+  using S = StagedRow<TI, BP>;
+#pragma unroll
+  for (int q = 0; q < S::B::nq; ++q)
+#pragma unroll
+    for (int i = 0; i < S::words; ++i) {
+      const int c = q * S::words + i;
+      if constexpr (std::is_same<TI, float>::value) {
+        o[c] = __uint_as_float(r.w[q][i]);
+      } else {
+        o[2 * c] = __uint_as_float(r.w[q][i] << 16);
+        o[2 * c + 1] = __uint_as_float(r.w[q][i] & 0xffff0000u);
+      }
+    }
+}
+
+// A run of RL consecutive offsets whose first has mask bit k0: p is the staged
+// row that the thread's first row reads at the first offset.  An entry that is
+// present is added as fma(v, 1, acc), one that is not as fma(v, 0, acc): acc
+// itself for every finite v.  (Predicated adds compile to adds and selects on
+// the half-rate ALU pipe: 76 us packed and 72 us scalar for the float product
+// at 128^3, where multiply-adds took 70.)  A non-finite v of an absent
+// entry makes acc NaN: a warp that ends with a NaN sums its rows again by
+// plain adds of what is present, gathered from global memory.
+template <int RL, typename TI, int BP>
+__device__ __forceinline__ void staged_run(const unsigned char *p, int rot, const unsigned (&mk)[kBlkRows], int k0,
+                                           StagedAcc<TI, BP> (&acc)[kBlkRows]) {
+  constexpr int rb = BlockTraits<TI, BP>::row_bytes;
+  StagedRow<TI, BP> r[RL + kBlkRows - 1];
+#pragma unroll
+  for (int i = 0; i < RL + kBlkRows - 1; ++i) r[i].load(p + i * rb, rot);
+#pragma unroll
+  for (int j = 0; j < kBlkRows; ++j) {
+    const unsigned m = mk[j] >> k0;
+#pragma unroll
+    for (int t = 0; t < RL; ++t) acc[j].fma(r[j + t], (m & (1u << t)) != 0);   // ascending offsets
+  }
+}
+
+// waits for the first phase of an mbarrier; false after 2^16 tries (each of
+// them a hardware wait of its own), which the copies of a block never need:
+// the caller then reads global memory instead
+__device__ __forceinline__ bool staged_wait(unsigned bar32) {
+  for (int tries = 0; tries < (1 << 16); ++tries) {
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok)
+                 : "r"(bar32)
+                 : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// Descriptor of a block (kBlkDesc ints): [0] ranges, [1] runs, [2] staged row of
+// the block's row 0; then per range {first row relative to the block's, rows,
+// staged row}; then per run: staged row | length << 16 | first mask bit << 18.
+// mask: a row's entries among the block's offsets, or bit 31 for a row without
+// short entries here (long rows, rows past the end).
+template <typename TI, typename TT, int BP, int MODE>
+__global__ void __launch_bounds__(kBlkThreads, BlockTraits<TI, BP>::min_blocks)
+k_spmm_block(const LapView L, const SpmmDev a, const int32_t *__restrict__ desc, const unsigned *__restrict__ mask) {
+  using B = BlockTraits<TI, BP>;
+  constexpr int rb = B::row_bytes;
+  extern __shared__ __align__(16) unsigned char staged[];
+  __shared__ int sd[kBlkDesc];
+  __shared__ __align__(8) unsigned long long bar;
+  if (a.done && *a.done) return;
+  const int tid = threadIdx.x, T = blockDim.x;
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * (kBlkRows * T);
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(&bar))) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int i = tid; i < kBlkDesc; i += T) sd[i] = __ldg(desc + static_cast<int64_t>(blockIdx.x) * kBlkDesc + i);
+  unsigned mk[kBlkRows];   // padded to whole blocks
+#pragma unroll
+  for (int j = 0; j < kBlkRows; ++j) mk[j] = __ldcs(mask + r0 + kBlkRows * tid + j);
+  __syncthreads();
+  const int nrange = sd[0], nrun = sd[1];
+  const unsigned char *x = static_cast<const unsigned char *>(a.x);
+  const unsigned bar32 = static_cast<unsigned>(__cvta_generic_to_shared(&bar));
+  for (int k = 0; k < nrange; ++k) {
+    const int rows = sd[4 + 3 * k];
+    const int64_t g0 = r0 + sd[3 + 3 * k];                       // even, as is the range's staged row
+    const int head = g0 < 0 ? static_cast<int>(-g0 < rows ? -g0 : rows) : 0;       // rows before the matrix
+    const int tail = L.n - g0 < rows ? static_cast<int>(L.n - g0 > head ? L.n - g0 : head) : rows;   // rows inside end here
+    unsigned char *own = staged + sd[5 + 3 * k] * rb;
+    const int bytes = (tail - head) * rb;                        // an odd row of 8 (24) bytes is left over
+    if (tid == k && bytes >= 16) {                               // one thread a range
+      asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar32), "r"(bytes & ~15) : "memory");
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                       static_cast<unsigned>(__cvta_generic_to_shared(own)) + head * rb),
+                   "l"(x + (g0 + head) * rb), "r"(bytes & ~15), "r"(bar32)
+                   : "memory");
+    }
+    if (tid == k && (bytes & 15))
+      *reinterpret_cast<uint2 *>(own + tail * rb - 8) = *reinterpret_cast<const uint2 *>(x + (g0 + tail) * rb - 8);
+    // rows outside the matrix are zeros (absent entries multiply them by zero)
+    for (int c = 8 * tid; c < head * rb; c += 8 * T) *reinterpret_cast<uint2 *>(own + c) = make_uint2(0u, 0u);
+    for (int c = tail * rb + 8 * tid; c < rows * rb; c += 8 * T) *reinterpret_cast<uint2 *>(own + c) = make_uint2(0u, 0u);
+  }
+  __syncthreads();   // expectations and plain stores first
+  if (tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar32) : "memory");
+  const bool landed = staged_wait(bar32);
+  const int rot = B::nq == 2 ? (tid >> 2) & 1 : (B::nq == 4 ? (tid >> 1) & 3 : 0);
+  const unsigned char *mine = staged + tid * (kBlkRows * rb);
+  const int *runs = sd + 3 + 3 * nrange;
+  StagedAcc<TI, BP> acc[kBlkRows];
+#pragma unroll
+  for (int j = 0; j < kBlkRows; ++j) acc[j].zero();
+  for (int k = 0; k < nrun; ++k) {
+    const int e = runs[k];
+    const unsigned char *p = mine + (e & 0xffff) * rb;
+    const int len = (e >> 16) & 3, k0 = e >> 18;
+    if (len == 3) staged_run<3, TI, BP>(p, rot, mk, k0, acc);
+    else if (len == 2) staged_run<2, TI, BP>(p, rot, mk, k0, acc);
+    else staged_run<1, TI, BP>(p, rot, mk, k0, acc);
+  }
+  float sum[kBlkRows][BP], chk = 0.f;   // chk: NaN if any sum is (or infinities cancel)
+#pragma unroll
+  for (int j = 0; j < kBlkRows; ++j) {
+    acc[j].get(sum[j]);
+#pragma unroll
+    for (int c = 0; c < BP; ++c) chk += sum[j][c];
+  }
+  if (__any_sync(kFull, chk != chk || !landed)) {
+#pragma unroll
+    for (int j = 0; j < kBlkRows; ++j)
+#pragma unroll
+      for (int c = 0; c < BP; ++c) sum[j][c] = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < nrun; ++k) {
+      const int e = runs[k], base = e & 0xffff;
+      int off = 0;   // the run's first offset, from the range that holds its staged row
+      for (int q = 0; q < nrange; ++q)
+        if (base >= sd[5 + 3 * q] && base < sd[5 + 3 * q] + sd[4 + 3 * q]) off = base - sd[5 + 3 * q] + sd[3 + 3 * q];
+#pragma unroll
+      for (int j = 0; j < kBlkRows; ++j)
+        for (int t = 0; t < ((e >> 16) & 3); ++t) {
+          if (!((mk[j] >> ((e >> 18) + t)) & 1u)) continue;
+          StagedRow<TI, BP> r;
+          float v[BP];
+          r.load(x + (r0 + kBlkRows * tid + j + t + off) * rb, rot);
+          staged_values<TI, BP>(r, v);
+#pragma unroll
+          for (int c = 0; c < BP; ++c) sum[j][c] += v[c];
+        }
+    }
+    if (!landed) (void)staged_wait(bar32);   // copies still in flight write to this block's memory
+  }
+#pragma unroll
+  for (int j = 0; j < kBlkRows; ++j) {
+    if (mk[j] >> 31) continue;   // a long row, or past the end
+    float ord[BP], xi[BP];
+#pragma unroll
+    for (int c = 0; c < BP; ++c) {   // columns back in order
+      ord[c] = sum[j][c];
+      if constexpr (B::nq == 2) {
+        ord[c] = rot ? sum[j][(c + BP / 2) % BP] : sum[j][c];
+      } else if constexpr (B::nq == 4) {
+        constexpr int w = BP / 4;   // row chunk c / w is lane chunk (c / w - rot) mod 4
+        const float even = (rot & 2) ? sum[j][(c + 2 * w) % BP] : sum[j][c];
+        const float odd = (rot & 2) ? sum[j][(c + w) % BP] : sum[j][(c + 3 * w) % BP];
+        ord[c] = (rot & 1) ? odd : even;
+      }
+    }
+    StagedRow<TI, BP> r;
+    if (landed) r.load(mine + (sd[2] + j) * rb, 0);
+    else r.load(x + (r0 + kBlkRows * tid + j) * rb, 0);
+    staged_values<TI, BP>(r, xi);
+    spmm_epilogue<SPHYNX_COMBINATORIAL, TI, TT, BP, MODE>(L, a, r0 + kBlkRows * tid + j, xi, ord);
+  }
+}
+
+// launches the staged-block kernel when this product qualifies
+template <int LAP, typename TI, typename TT, int BP, bool W, int MODE>
+bool spmm_launch_block(sphynx_graph *g, const LapView &L, const SpmmDev &a) {
+  if constexpr (W || LAP == SPHYNX_NORMALIZED || std::is_same<TI, double>::value || BP == 1) {
+    return false;
+  } else {
+    const SpmmPlan &p = g->plan;
+    const size_t smem = static_cast<size_t>(p.blk_staged_rows) * BlockTraits<TI, BP>::row_bytes;
+    if (p.blk_threads == 0 || a.act_blocks || smem > kBlkSmemMax || reinterpret_cast<uintptr_t>(a.x) % 16) return false;
+    SPX_CUDA(cudaFuncSetAttribute(k_spmm_block<TI, TT, BP, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(kBlkSmemMax)));
+    const int64_t rows = static_cast<int64_t>(kBlkRows) * p.blk_threads;
+    k_spmm_block<TI, TT, BP, MODE><<<static_cast<unsigned>((g->n + rows - 1) / rows), p.blk_threads, smem, g->stream>>>(
+        L, a, p.blk_desc.as<int32_t>(), p.blk_mask.as<unsigned>());
+    return true;
+  }
+}
+
 // Medium rows (kShortDeg < degree <= med_max), sorted by degree at create: a
 // group of G lanes per row, G the smallest power of two that leaves each lane
 // at most kGroupPerLane entries (G = 32 above 32 kGroupPerLane entries), and
@@ -1025,9 +1342,9 @@ void spmm_launch_t(sphynx_graph *g, const SpmmDev &a) {
       const float *swp = a.coef_sell ? a.coef_sell : p.sell_w.as<float>();
       const int64_t *sp = p.sell_ptr.as<int64_t>();
       const uint8_t *sd = p.sell_deg.as<uint8_t>();
-      bool launched = false;
+      bool launched = p.variant == kSellPattern && spmm_launch_block<LAP, TI, TT, BP, W, MODE>(g, L, a);
       if constexpr (!W) {
-        if (p.variant == kSellPattern) {
+        if (p.variant == kSellPattern && !launched) {
           const int64_t *pc = p.pat_cptr.as<int64_t>();
           const int16_t *pcl = p.pat_col.as<int16_t>();
           if (p.pat_all)
