@@ -33,38 +33,83 @@ constexpr int kSmallThreads = 256;
 
 // ---- cooperative building blocks (all threads of the CTA call them) --------
 
+// 1 / d for a positive normal d: the hardware's approximation (20 bits) and two
+// Newton steps, four dependent FP64 operations (the division takes more than
+// twice that, and an FP64 instruction of a warp occupies its quarter of the SM
+// for 64 cycles)
+__device__ __forceinline__ double recip_newton(double d) {
+  double x;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
+  x = fma(x, fma(-d, x, 1.0), x);
+  return fma(x, fma(-d, x, 1.0), x);
+}
+
+// element t of the row-major upper triangle of an m x m matrix
+__device__ __forceinline__ void upper_element(int t, int m, int &i, int &j) {
+  i = 0;
+  while (t >= m - i) {
+    t -= m - i;
+    ++i;
+  }
+  j = i + t;
+}
+
 // In-place Cholesky of the leading m x m of B (ld): on success the upper
 // triangle holds R with B = R^T R.  Returns the smallest pivot (R_kk^2) or
-// a negative value if a pivot was not positive.
+// a negative value if a pivot was not positive.  A thread keeps its elements
+// of the upper triangle in registers and eliminates with unscaled rows
+// (B_ij -= B_ki B_kj / d_k); the thread that forms the next pivot also forms its
+// reciprocal, so a step has one barrier, and the rows are scaled by
+// 1 / sqrt(d_k) together at the end: 16.5 -> 10.6 us at m = 21 (scaled rows, three
+// barriers a step before).  `scratch` needs 2 m + 2 doubles.
 __device__ double chol_upper(double *B, int ld, int m, double *scratch) {
+  constexpr int kItems = (kMaxM * (kMaxM + 1) / 2 + kSmallThreads - 1) / kSmallThreads;   // 5
   const int tid = threadIdx.x;
-  if (tid == 0) scratch[0] = INFINITY;
+  double *piv = scratch + 2, *rec = scratch + 2 + m;
+  const int total = m * (m + 1) / 2;
+  int ei[kItems], ej[kItems];
+  double v[kItems];
+#pragma unroll
+  for (int u = 0; u < kItems; ++u) {
+    const int t = tid + u * kSmallThreads;
+    ei[u] = -1;
+    ej[u] = 0;
+    if (t < total) {
+      upper_element(t, m, ei[u], ej[u]);
+      v[u] = B[ei[u] * ld + ej[u]];
+    }
+  }
+  if (tid == 0) {
+    piv[0] = v[0];
+    rec[0] = recip_newton(v[0]);
+  }
   __syncthreads();
+  double mn = INFINITY;
   for (int k = 0; k < m; ++k) {
-    if (tid == 0) {
-      const double d = B[k * ld + k];
-      if (!(d > 0.0)) {
-        scratch[0] = -1.0;
-      } else {
-        if (d < scratch[0]) scratch[0] = d;
-        const double r = rsqrt(d);   // 1 / R_kk; R_kk = d r (the row below is scaled by r, not divided)
-        B[k * ld + k] = d * r;
-        scratch[1] = r;
+    const double d = piv[k];
+    if (!(d > 1e-30)) return -1.0;   // uniform; the scaled Gram has a unit diagonal
+    mn = d < mn ? d : mn;
+    const double r = rec[k];
+#pragma unroll
+    for (int u = 0; u < kItems; ++u) {
+      if (u * kSmallThreads >= total) break;
+      if (ei[u] <= k) continue;
+      v[u] = fma(-(B[k * ld + ei[u]] * r), B[k * ld + ej[u]], v[u]);
+      if (ei[u] == k + 1) {
+        B[ei[u] * ld + ej[u]] = v[u];
+        if (ej[u] == k + 1) {        // the next pivot
+          piv[k + 1] = v[u];
+          rec[k + 1] = recip_newton(v[u]);
+        }
       }
     }
     __syncthreads();
-    if (scratch[0] < 0.0) return -1.0;
-    const double rinv = scratch[1];
-    for (int j = k + 1 + tid; j < m; j += blockDim.x) B[k * ld + j] *= rinv;
-    __syncthreads();
-    const int rem = m - k - 1;
-    for (int idx = tid; idx < rem * rem; idx += blockDim.x) {
-      const int i = k + 1 + idx / rem, j = k + 1 + idx % rem;
-      if (j >= i) B[i * ld + j] -= B[k * ld + i] * B[k * ld + j];
-    }
-    __syncthreads();
   }
-  const double mn = scratch[0];
+  for (int k = tid; k < m; k += blockDim.x) rec[k] = rsqrt(piv[k]);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kItems; ++u)
+    if (ei[u] >= 0) B[ei[u] * ld + ej[u]] *= rec[ei[u]];
   __syncthreads();
   return mn;
 }
@@ -279,17 +324,18 @@ struct RRSmem {
   float A32[kMaxM * (kMaxM + 1)];  // float copies for the float-started solve (odd leading dimension)
   float V32[kMaxM * (kMaxM + 1)];
   float cs32[2 * kMaxM];
+  float sel32[kMaxM];        // float reciprocal pivots of the refined path
+  int top;
   int pq32[2 * kMaxM];
   double d[kMaxM];
   double rinv[kMaxM];        // reciprocal Cholesky pivots
   double cs[2 * kMaxM];      // Jacobi rotations (c, s) and pairs (p, q)
   int pq[2 * kMaxM];
-  double qa[SPHYNX_MAX_NEV], qb[SPHYNX_MAX_NEV];
-  double scratch[4];
+  double qa[SPHYNX_MAX_NEV];
+  double scratch[2 * kMaxM + 2];   // Cholesky pivots and reciprocals
   int idx[kMaxM];            // active column -> full index
   int order[kMaxM];
   int keep[kMaxM];
-  int sel[SPHYNX_MAX_NEV];
   unsigned amask[2];         // active columns, one ballot per warp
   int m, m2, fail, svqb;
 };
@@ -337,6 +383,411 @@ __device__ void eig_sym(RRSmem &S, double *A, double *V, int m, bool float_start
     A[i * L + j] = i == j ? S.P0[i * L + i] : 0.0;
   }
   __syncthreads();
+}
+
+// Results of a Rayleigh-Ritz step: S.T (m x nev, scaled coordinates) and S.qa
+// to the outputs; all threads call it.
+__device__ void rr_write(RRSmem &S, int m, int M, int ld, int nev, SolverState *st, double *y64, void *yt, int yt_f32,
+                         double *theta_out, int *svqb_out) {
+  const int L = kMaxM, tid = threadIdx.x;
+  for (int e = tid; e < M * ld; e += blockDim.x) {
+    if (y64) y64[e] = 0.0;
+    if (yt) {
+      if (yt_f32) static_cast<float *>(yt)[e] = 0.f;
+      else static_cast<double *>(yt)[e] = 0.0;
+    }
+  }
+  __syncthreads();
+  // Y = D y (rows of inactive columns stay zero)
+  for (int e = tid; e < m * nev; e += blockDim.x) {
+    const int i = e / nev, c = e % nev;
+    const double v = S.d[i] * S.T[i * L + c];
+    const int o = S.idx[i] * ld + c;
+    if (y64) y64[o] = v;
+    if (yt) {
+      if (yt_f32) static_cast<float *>(yt)[o] = static_cast<float>(v);
+      else static_cast<double *>(yt)[o] = v;
+    }
+  }
+  if (tid < nev) {
+    const double th = S.qa[tid];
+    if (st) st->theta[tid] = th;
+    if (theta_out) theta_out[tid] = th;
+  }
+  if (tid == 0) {
+    if (st) st->svqb_steps += S.svqb;
+    if (svqb_out) *svqb_out = S.svqb;
+  }
+}
+
+// ---- refined Rayleigh-Ritz ---------------------------------------------------
+// The wanted eigenpairs of A x = theta B x (A, B the scaled Gram matrices, B of
+// unit diagonal) to FP64 accuracy from a float eigendecomposition, by the
+// refinement of Ogita and Aishima ("Iterative refinement for symmetric
+// eigenvalue decomposition", 2018) in B-inner products and for the nev wanted
+// columns only: with X the current basis, S = X^T A X, R = I - X^T B X and
+// theta_j = S_jj / (1 - R_jj),
+//   x_j += sum_i x_i E_ij,  E_ij = (S_ij + theta_j R_ij) / (theta_j - theta_i),
+// E_jj = R_jj / 2: a step costs 5 m^2 nev FP64 multiply-adds and squares the
+// error (a float eigendecomposition's 1e-6 -> 1e-11 -> below rounding).  FP64 is
+// what this kernel is short of (2 lanes a clock on the one SM it runs on): a
+// sweep of FP64 Jacobi rotations, of which eight (or three, float-started) were
+// needed, takes as long as a dozen such steps.  Pairs too close for the quotient only keep
+// their orthogonality in the steps; if both are wanted a small FP64 Jacobi
+// solve on the nev x nev projection separates them, if not the caller's general
+// path runs.  The whole kernel at m = 21, nev = 7: 273 -> 82 us from float blocks,
+// 396 -> 95 us in FP64; m = 12, nev = 4: 124 and 165 -> 40 us.  Half of it is now the
+// float eigendecomposition (one warp, latency).
+
+// Float eigendecomposition of the pencil by one warp, lane j owning column j in
+// registers (m <= MP <= 32): W = R^{-T} A R^{-1} by two triangular solves, a
+// Gershgorin shift makes it positive definite, W + s I = L L^T, and one-sided
+// Jacobi rotations of L's columns (Hestenes; round-robin pairs, partner columns
+// read by shuffles) end in L J = U Sigma: U's columns are W's eigenvectors.  No
+// barriers and no shared traffic inside a sweep.  Returns X = R^{-1} U in
+// columns of x32 (ld), eigenvalues in lam.  Sweeps stop once every pair was
+// within 1e-3 of orthogonal before its rotation (then 1e-6 after it).
+template <int MP>
+__device__ void warp_pencil32(const double *A, int ld, int m, double ascale, const float *x32, int ldx,
+                              float *lam, int *pq) {
+  const int lane = threadIdx.x & 31;
+  const bool in = lane < m;
+  float own[MP];
+  // own = column lane of A; then R^{-T} twice (W is symmetric: transpose between)
+#pragma unroll
+  for (int i = 0; i < MP; ++i) own[i] = in && i < m ? static_cast<float>(A[i * ld + lane] * ascale) : 0.f;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+    for (int i = 0; i < MP; ++i) {
+      if (i < m) {
+        own[i] *= x32[i * ldx + i];   // 1 / R_ii
+#pragma unroll
+        for (int k = i + 1; k < MP; ++k)
+          if (k < m) own[k] = fmaf(-x32[i * ldx + k], own[i], own[k]);
+      }
+    }
+    if (pass == 0) {   // transpose through lam's neighbour buffer
+      float *t = lam + 32;
+#pragma unroll
+      for (int i = 0; i < MP; ++i)
+        if (i < m && in) t[lane * ldx + i] = own[i];
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < MP; ++i)
+        if (i < m && in) own[i] = t[i * ldx + lane];
+      __syncwarp();
+    }
+  }
+  // rows and columns by decreasing diagonal: the factor's columns start closer
+  // to orthogonal (a third fewer sweeps)
+  float *t = lam + 32;
+  float dia = 0.f;
+#pragma unroll
+  for (int i = 0; i < MP; ++i) {
+    if (i == lane) dia = own[i];
+    if (i < m && in) t[lane * ldx + i] = own[i];
+  }
+  int rank = 0;
+  for (int j = 0; j < m; ++j) {
+    const float dj = __shfl_sync(0xffffffffu, dia, j);
+    rank += (dj > dia || (dj == dia && j < lane)) ? 1 : 0;
+  }
+  if (in) pq[rank] = lane;
+  __syncwarp();
+  const int mycol = in ? pq[lane] : 0;
+  float rad = 0.f;
+#pragma unroll
+  for (int i = 0; i < MP; ++i) {
+    own[i] = in && i < m ? t[mycol * ldx + pq[i]] : 0.f;
+    rad += i == lane ? 0.f : fabsf(own[i]);
+    if (i == lane) dia = own[i];
+  }
+  // Gershgorin shift: every eigenvalue of W + s I at least 1e-3 of the largest row sum
+  float lo = in ? dia - rad : 0.f, hi = in ? fabsf(dia) + rad : 0.f;
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  const float shift = (lo < 0.f ? -lo : 0.f) + 1e-3f * hi;
+#pragma unroll
+  for (int i = 0; i < MP; ++i)
+    if (i == lane) own[i] = in ? own[i] + shift : 1.f;
+  // Cholesky, lane j keeping column j of L
+#pragma unroll
+  for (int k = 0; k < MP; ++k) {
+    const float r = rsqrtf(fmaxf(__shfl_sync(0xffffffffu, own[k], k), 1e-30f));
+    const float mine = own[k] * r;   // L_{lane,k} by symmetry
+#pragma unroll
+    for (int i = k; i < MP; ++i) {
+      const float li = __shfl_sync(0xffffffffu, own[i], k) * r;
+      if (lane > k) own[i] = fmaf(-li, mine, own[i]);
+      else if (lane == k) own[i] = li;
+    }
+    if (lane > k) own[k] = 0.f;
+  }
+  // one-sided Jacobi
+  const int mp = m + (m & 1);
+  for (int sweep = 0; sweep < 12; ++sweep) {
+    float nn = 0.f, worst = 0.f;
+#pragma unroll
+    for (int i = 0; i < MP; ++i) nn = fmaf(own[i], own[i], nn);
+    // round r pairs i with (r - i) mod (mp - 1); the one that would meet itself meets mp - 1
+    int q = lane >= mp ? lane : (lane == mp - 1 ? 0 : (lane == 0 ? 0 : mp - 1 - lane));
+    for (int r = 0; r < mp - 1; ++r) {
+      const int w = lane < mp - 1 && q == lane ? mp - 1 : q;
+      float oth[MP], d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
+#pragma unroll
+      for (int i = 0; i < MP; ++i) oth[i] = __shfl_sync(0xffffffffu, own[i], w);
+      const float no = __shfl_sync(0xffffffffu, nn, w);
+#pragma unroll
+      for (int i = 0; i < MP; i += 4) {
+        d0 = fmaf(own[i], oth[i], d0);
+        d1 = fmaf(own[i + 1], oth[i + 1], d1);
+        d2 = fmaf(own[i + 2], oth[i + 2], d2);
+        d3 = fmaf(own[i + 3], oth[i + 3], d3);
+      }
+      const float pq2 = 2.f * ((d0 + d1) + (d2 + d3));
+      const bool first = lane < w;
+      const float df = first ? no - nn : nn - no;          // a_qq - a_pp
+      const float h2 = fmaf(df, df, pq2 * pq2), an = nn * no;
+      // tan of the smaller angle: 2 a_pq / (d +- sqrt(d^2 + 4 a_pq^2))
+      float t1 = __fdividef(pq2, df + copysignf(h2 * rsqrtf(h2), df));
+      if (w == lane || !(pq2 * pq2 > 1e-15f * an)) t1 = 0.f;
+      const float c = rsqrtf(fmaf(t1, t1, 1.f)), s = t1 * c;
+      worst = fmaxf(worst, w == lane ? 0.f : __fdividef(pq2 * pq2, an));
+      const float so = first ? -s : s;
+#pragma unroll
+      for (int i = 0; i < MP; ++i) own[i] = fmaf(so, oth[i], c * own[i]);
+      nn = fmaf(first ? -0.5f * t1 : 0.5f * t1, pq2, nn);
+      if (lane < mp - 1) q = q + 1 == mp - 1 ? 0 : q + 1;
+      else if (lane == mp - 1) q = q + mp / 2 >= mp - 1 ? q + mp / 2 - (mp - 1) : q + mp / 2;
+    }
+    if (__all_sync(0xffffffffu, worst < 4e-6f)) break;
+  }
+  float nn = 0.f;
+#pragma unroll
+  for (int i = 0; i < MP; ++i) nn = fmaf(own[i], own[i], nn);
+  const float inv = rsqrtf(fmaxf(nn, 1e-30f));
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < MP; ++i)
+    if (i < m && in) t[pq[i] * ldx + lane] = own[i] * inv;   // rows back in order
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < MP; ++i) own[i] = i < m && in ? t[i * ldx + lane] : 0.f;
+  // x = R^{-1} u
+#pragma unroll
+  for (int i = MP - 1; i >= 0; --i) {
+    if (i < m) {
+      own[i] *= x32[i * ldx + i];
+#pragma unroll
+      for (int k = 0; k < MP; ++k)
+        if (k < i) own[k] = fmaf(-x32[k * ldx + i], own[i], own[k]);
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < MP; ++i)
+    if (i < m && in) t[i * ldx + lane] = own[i];
+  if (in) lam[lane] = nn - shift;
+}
+
+// P0 = Q0 X_w and P1 = Q1 X_w (TRANS: Q^T X_w with one matrix and two blocks,
+// P0 = X^T Y0, P1 = X^T Y1): 2 m nev dots of length m in one pass of the threads
+template <bool TRANS>
+__device__ void pair_product(const double *Q0, const double *Q1, const double *Y0, const double *Y1, int ld, double *P0,
+                             double *P1, int m, int nev) {
+  for (int idx = threadIdx.x; idx < 2 * m * nev; idx += blockDim.x) {
+    const bool second = idx >= m * nev;
+    const int e = second ? idx - m * nev : idx;
+    const int i = e / nev, j = e - i * nev;
+    const double *q = (second ? Q1 : Q0) + (TRANS ? i : i * ld), *y = (second ? Y1 : Y0) + j;
+    const int qs = TRANS ? ld : 1;
+    double s0 = 0.0, s1 = 0.0;
+    int k = 0;
+    for (; k + 1 < m; k += 2) {
+      s0 = fma(q[k * qs], y[k * ld], s0);
+      s1 = fma(q[(k + 1) * qs], y[(k + 1) * ld], s1);
+    }
+    if (k < m) s0 = fma(q[k * qs], y[k * ld], s0);
+    (second ? P1 : P0)[i * ld + j] = s0 + s1;
+  }
+}
+
+// S.A, S.Bh: scaled Gram matrices, S.B: R with Bh = R^T R.  On success S.V's
+// leading nev columns hold the wanted vectors (B-orthonormal, ascending),
+// S.qa the values; false (uniform): nothing usable, run the general path.
+__device__ bool rr_refined(RRSmem &S, int m, int nev) {
+  const int L = kMaxM, tid = threadIdx.x;
+  constexpr int L32 = kMaxM + 1;
+  // largest |A_ij| by exponent; reject what float cannot hold
+  int top = 0;
+  for (int e = tid; e < m * m; e += blockDim.x) {
+    const int hi = __double2hiint(S.A[(e / m) * L + e % m]) & 0x7fffffff;
+    top = hi > top ? hi : top;
+    const int i = e / m, j = e % m;   // float R, reciprocal diagonal
+    S.A32[i * L32 + j] = j > i ? static_cast<float>(S.B[i * L + j]) : 0.f;
+  }
+  for (int i = tid; i < m; i += blockDim.x) S.sel32[i] = 1.f / static_cast<float>(S.B[i * L + i]);
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (tid == 0) S.top = 0;
+  __syncthreads();
+  if ((tid & 31) == 0) atomicMax(&S.top, top);
+  for (int i = tid; i < m; i += blockDim.x) S.A32[i * L32 + i] = S.sel32[i];
+  __syncthreads();
+  const int ex = S.top >> 20;   // biased exponent of the largest entry
+  if (ex < 64 || ex > 1983) return false;
+  const double ascale = __hiloint2double((2046 - ex) << 20, 0);   // 2^(1023 - ex)
+  if (tid < 32) {
+    float *lam = S.V32;          // 32 values, then the m x m output
+    if (m <= 12) warp_pencil32<12>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32);
+    else if (m <= 24) warp_pencil32<24>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32);
+    else warp_pencil32<32>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32);
+  }
+  __syncthreads();
+  const float *lam = S.V32, *x32 = S.V32 + 32;
+  for (int i = tid; i < m; i += blockDim.x) {   // ascending order, stable
+    const float li = lam[i];
+    int rank = 0;
+    for (int j = 0; j < m; ++j) rank += (lam[j] < li || (lam[j] == li && j < i)) ? 1 : 0;
+    S.order[rank] = i;
+    S.cs[rank] = static_cast<double>(li) / ascale;   // theta of every column, in order
+  }
+  __syncthreads();
+  for (int e = tid; e < m * m; e += blockDim.x) {
+    const int i = e / m, j = e % m;
+    S.V[i * L + j] = static_cast<double>(x32[i * L32 + S.order[j]]);
+  }
+  __syncthreads();
+  int close = 0;
+  for (int step = 0;; ++step) {
+    pair_product<false>(S.A, S.Bh, S.V, S.V, L, S.P0, S.P1, m, nev);
+    __syncthreads();
+    pair_product<true>(S.V, S.V, S.P0, S.P1, L, S.W, S.P2, m, nev);   // S_ij, (X^T B X)_ij
+    __syncthreads();
+    if (tid < nev) {
+      const double r = 1.0 - S.P2[tid * L + tid];
+      S.cs[tid] = S.W[tid * L + tid] * (1.0 + r + r * r);
+    }
+    __syncthreads();
+    int big = 0, bad = 0, pair = 0;
+    for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      const double rij = (i == j ? 1.0 : 0.0) - S.P2[i * L + j];
+      double e = 0.5 * rij;
+      if (i != j) {
+        const float num = static_cast<float>((S.W[i * L + j] + S.cs[j] * rij) * ascale);
+        const float gap = static_cast<float>((S.cs[j] - S.cs[i]) * ascale);
+        if (fabsf(num) <= 1e-3f * fabsf(gap)) {
+          e = static_cast<double>(num / gap);
+        } else if (fabsf(num) > 4e-16f * m) {           // unresolved, and not rounding
+          if (i < nev) pair = 1;
+          else bad = 1;
+        }
+      }
+      if (!(fabs(e) < 0.05)) bad = 1;                   // the float basis is no start (NaN included)
+      if (fabsf(static_cast<float>(e)) > 1e-11f) big = 1;
+      S.P0[i * L + j] = e;
+    }
+    const int flags = __syncthreads_or(big | (bad << 1) | (pair << 2));
+    if ((flags & 2) || step == 5) return false;
+    for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      double s0 = S.V[i * L + j], s1 = 0.0;
+      int k = 0;
+      for (; k + 1 < m; k += 2) {
+        s0 = fma(S.V[i * L + k], S.P0[k * L + j], s0);
+        s1 = fma(S.V[i * L + k + 1], S.P0[(k + 1) * L + j], s1);
+      }
+      if (k < m) s0 = fma(S.V[i * L + k], S.P0[k * L + j], s0);
+      S.P1[i * L + j] = s0 + s1;
+    }
+    __syncthreads();
+    for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      S.V[i * L + j] = S.P1[i * L + j];
+    }
+    __syncthreads();
+    close = flags & 4;
+    if (!(flags & 1)) break;
+  }
+  if (close) {
+    // wanted values too close for the quotient: FP64 Jacobi on the projection
+    pair_product<false>(S.A, S.Bh, S.V, S.V, L, S.P0, S.P1, m, nev);
+    __syncthreads();
+    for (int idx = tid; idx < nev * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      double acc = 0.0;
+      for (int k = 0; k < m; ++k) acc = fma(S.V[k * L + i], S.P0[k * L + j], acc);
+      S.W[i * L + j] = acc;
+    }
+    __syncthreads();
+    symmetrize(S.W, L, nev);
+    jacobi_eig<double>(S.W, L, S.P2, L, nev, S.cs, S.pq);
+    sort_diag(S.W, L, nev, S.order);
+    for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      double acc = 0.0;
+      for (int k = 0; k < nev; ++k) acc = fma(S.V[i * L + k], S.P2[k * L + S.order[j]], acc);
+      S.P1[i * L + j] = acc;
+    }
+    if (tid < nev) S.qa[tid] = S.W[S.order[tid] * L + S.order[tid]];
+    __syncthreads();
+    for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      S.V[i * L + j] = S.P1[i * L + j];
+    }
+  } else if (tid < nev) {
+    S.qa[tid] = S.cs[tid];
+  }
+  __syncthreads();
+  // the order may have changed among values equal in float
+  bool sorted = true;
+  for (int j = 0; j + 1 < nev; ++j) sorted = sorted && S.qa[j] <= S.qa[j + 1];
+  if (!sorted) {
+    if (tid < nev) {
+      int rank = 0;
+      for (int j = 0; j < nev; ++j) rank += (S.qa[j] < S.qa[tid] || (S.qa[j] == S.qa[tid] && j < tid)) ? 1 : 0;
+      S.order[rank] = tid;
+      S.cs[rank] = S.qa[tid];
+    }
+    __syncthreads();
+    for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      S.P1[i * L + j] = S.V[i * L + S.order[j]];
+    }
+    __syncthreads();
+    for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+      const int i = idx / nev, j = idx - (idx / nev) * nev;
+      S.V[i * L + j] = S.P1[i * L + j];
+    }
+    if (tid < nev) S.qa[tid] = S.cs[tid];
+    __syncthreads();
+  }
+  // sign as in the general path: w = R x, largest |entry| positive, first on ties
+  for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+    const int i = idx / nev, j = idx - (idx / nev) * nev;
+    double acc = 0.0;
+    for (int k = i; k < m; ++k) acc = fma(S.B[i * L + k], S.V[k * L + j], acc);
+    S.P0[i * L + j] = acc;
+  }
+  __syncthreads();
+  if (tid < nev) {
+    double best = -1.0;
+    int bi = 0;
+    for (int k = 0; k < m; ++k) {
+      const double w = fabs(S.P0[k * L + tid]);
+      if (w > best) { best = w; bi = k; }
+    }
+    S.keep[tid] = S.P0[bi * L + tid] < 0.0 ? -1 : 1;
+  }
+  __syncthreads();
+  for (int idx = tid; idx < m * nev; idx += blockDim.x) {
+    const int i = idx / nev, j = idx - (idx / nev) * nev;
+    S.T[i * L + j] = S.V[i * L + j] * S.keep[j];
+  }
+  return true;
 }
 
 // One Rayleigh-Ritz step.  ga/gb: full M x M (device).  The active mask is
@@ -413,6 +864,11 @@ k_rayleigh_ritz(const double *ga, const double *gb, int M, int ld, int nev, doub
   __syncthreads();
   const double minpiv = chol_upper(S.B, L, m, S.scratch);
   int m2 = m;
+  // the refined path wants a basis that float arithmetic can orthogonalise
+  if (minpiv >= tau && minpiv >= 1e-4 && m >= 2 && m <= 32 && nev <= m && rr_refined(S, m, nev)) {
+    rr_write(S, m, M, ld, nev, st, y64, yt, yt_f32, theta_out, svqb_out);
+    return;
+  }
   if (minpiv >= tau) {
     tri_inv_upper(S.B, L, m, S.C, L, S.rinv);
   } else {
@@ -473,41 +929,8 @@ k_rayleigh_ritz(const double *ga, const double *gb, int M, int ld, int nev, doub
     for (int k = 0; k < m2; ++k) s += S.C[i * L + k] * S.V[k * L + col];
     S.T[i * L + c] = s * S.keep[c];
   }
-  if (tid < nev) {
-    S.sel[tid] = tid;
-    S.qa[tid] = S.W[S.order[tid] * L + S.order[tid]];
-    S.qb[tid] = 1.0;
-  }
-  __syncthreads();
-  for (int e = tid; e < M * ld; e += blockDim.x) {
-    if (y64) y64[e] = 0.0;
-    if (yt) {
-      if (yt_f32) static_cast<float *>(yt)[e] = 0.f;
-      else static_cast<double *>(yt)[e] = 0.0;
-    }
-  }
-  __syncthreads();
-  // Y = D y (rows of inactive columns stay zero)
-  for (int e = tid; e < m * nev; e += blockDim.x) {
-    const int i = e / nev, c = e % nev;
-    const int src = S.sel[c];
-    const double v = S.d[i] * S.T[i * L + src];
-    const int o = S.idx[i] * ld + c;
-    if (y64) y64[o] = v;
-    if (yt) {
-      if (yt_f32) static_cast<float *>(yt)[o] = static_cast<float>(v);
-      else static_cast<double *>(yt)[o] = v;
-    }
-  }
-  if (tid < nev) {
-    const double th = S.qa[S.sel[tid]];
-    if (st) st->theta[tid] = th;
-    if (theta_out) theta_out[tid] = th;
-  }
-  if (tid == 0) {
-    if (st) st->svqb_steps += S.svqb;
-    if (svqb_out) *svqb_out = S.svqb;
-  }
+  if (tid < nev) S.qa[tid] = S.W[S.order[tid] * L + S.order[tid]];
+  rr_write(S, m, M, ld, nev, st, y64, yt, yt_f32, theta_out, svqb_out);
 }
 
 // Harmonic Ritz values of the Lanczos tridiagonal T (Sec. 5.2 setup): the
