@@ -33,10 +33,18 @@ namespace sphynx {
 
 namespace {
 
-// rows per chunk: large enough that a CTA's reduction and its partial
+// Rows per chunk: at most kBatchChunk, so that a CTA's reduction and its partial
 // outputs are paid for by many rows (with 1024-row chunks, the 2000-graph
-// batch's 75,000 chunks made each reduction kernel launch-overhead-bound)
+// batch's 75,000 chunks made each reduction kernel launch-overhead-bound), and
+// few enough that the batch fills the GPU with four chunks an SM: a chunk's
+// FP64 sums run on one SM's FP64 pipe (24 graphs of 1,000 to 12,000 rows, K = 8:
+// 167 -> 50 to 56 ms a partition, one chunk a graph before).
 constexpr int kBatchChunk = 16384;
+constexpr int kBatchChunkMin = 256;
+int64_t batch_chunk_rows(int64_t n) {
+  const int64_t rows = (n / (4 * kSmCount) + kBatchChunkMin - 1) / kBatchChunkMin * kBatchChunkMin;
+  return std::max<int64_t>(kBatchChunkMin, std::min<int64_t>(rows, kBatchChunk));
+}
 constexpr int kGramRows = 64;       // rows staged per step of the batched Gram kernel
 constexpr int kGramThreads = 256;
 // iterations without a 10 % residual gain (at the float rounding floor) after
@@ -877,9 +885,10 @@ void batch_setup(sphynx_graph *g, const int64_t *h_gptr, int count) {
   std::vector<int32_t> cg;
   std::vector<int64_t> cb;
   std::vector<int32_t> c0(static_cast<size_t>(count) + 1);
+  const int64_t chunk = batch_chunk_rows(g->n);
   for (int q = 0; q < count; ++q) {
     c0[q] = static_cast<int32_t>(cg.size());
-    for (int64_t r = h_gptr[q]; r < h_gptr[q + 1]; r += kBatchChunk) {
+    for (int64_t r = h_gptr[q]; r < h_gptr[q + 1]; r += chunk) {
       cg.push_back(q);
       cb.push_back(r);
     }
