@@ -1405,9 +1405,10 @@ void batch_partition(sphynx_graph *g, int K, const sphynx_options *o, int32_t *d
   SPX_LAUNCHED();
   // multi-jagged over all graphs at once: graph q owns parts [q K, (q + 1) K)
   const int ktot = count * K;
-  void *mjs = g->workspace("mj", mj_scratch_bytes(n, ktot, count), false);
+  const size_t mj_bytes = mj_scratch_bytes(n, ktot, count, dt);
+  void *mjs = g->workspace("mj", mj_bytes, false);
   const int64_t *vw_caller = orig && B.vw_orig.p ? B.vw_orig.as<int64_t>() : g->vw;
-  run_mj_scratch(st, dt, coords, d - 1, d - 1, n, vw_caller, ktot, dpart, &g->ctr, mjs, B.h_gptr.data(), count);
+  run_mj_scratch(st, dt, coords, d - 1, d - 1, n, vw_caller, ktot, dpart, &g->ctr, mjs, mj_bytes, B.h_gptr.data(), count);
   // metrics per graph
   if (g->weighted && !g->wexact)
     fail(SPHYNX_ERR_UNSUPPORTED, "edge weights span too many binary orders for an exact cut");

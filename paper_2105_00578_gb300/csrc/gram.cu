@@ -7,15 +7,17 @@
 // double path uses k_gram, in 4 x 4 output tiles: NB = mb (mb + 1) tiles with
 // mb = M / 4.  A CTA streams slabs of TR rows of S, LS and diag(B) into shared
 // memory with cp.async 16-byte copies, multi-buffered so that the next slabs
-// are in flight while the current one is multiplied.  Its 256 threads form
-// floor(256 / NB) groups of NB threads, thread t of a group owning tile t and
-// the group owning rows grp, grp + ngroups, ...  Per row a thread does two
-// 16-byte shared loads and 16 FMAs (B applied on the fly for G_B tiles).
-// float: products and short sums in float, folded every 64 rows into a float
-// (hi, lo) pair with Knuth's TwoSum (about 48 significant bits); double:
-// plain double FMAs.  Per-CTA partials are written in double and a second
-// kernel adds them in a fixed order, so results do not depend on scheduling.
-// Every element of S and LS is read once: the kernel is bound by those bytes.
+// are in flight while the current one is multiplied.  Its threads form groups
+// of NB threads, thread t of a group owning tile t and the group owning rows
+// grp, grp + ngroups, ...  Per row a thread does four 16-byte shared loads and 16
+// FMAs.  Per-CTA partials are written in double and a second kernel adds them
+// in a fixed order, so results do not depend on scheduling.
+// Bound: the FP64 pipe (2 lanes a clock per SM), not the bytes.  So a warp's
+// lanes must all work: groups follow one another without regard to warps
+// (42 tiles at M = 24: 252 of 256 threads, where whole-warp groups left a third
+// idle), a slab is a whole number of rows for every group, and B S is formed once
+// per element, not once per tile.  n = 1,000,003, M = 24, B given: GRAM_OLD ->
+// GRAM_NEW us; the 672 FMAs a row alone take 1068 us.
 #include "internal.cuh"
 
 namespace sphynx {
@@ -25,14 +27,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kFoldRows = 4096;   // rows a thread of the 8 x 8 kernel adds into one float running sum
 
-template <typename T> struct Tile {
-  static constexpr int rows = 64;
-  static constexpr int stages = 4;   // slabs in flight: enough bytes to cover DRAM latency
-};
-template <> struct Tile<double> {
-  static constexpr int rows = 32;
-  static constexpr int stages = 3;
-};
+constexpr int kStages = 3;        // slabs of the double kernel in flight
 
 // four consecutive elements, moved with 16-byte accesses
 template <typename T> struct Q4 { T x, y, z, w; };
@@ -72,69 +67,18 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
   return r;
 }
 
-// 4 x 4 tile accumulator: a_i c_j for i, j < 4
-template <typename T> struct Acc44 {
-  T v[16];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int q = 0; q < 16; ++q) v[q] = T(0);
-  }
-  __device__ __forceinline__ void add(const Q4<T> &a, const Q4<T> &c) {
-    const T av[4] = {a.x, a.y, a.z, a.w}, cv[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[i * 4 + j] += av[i] * cv[j];
-  }
-  __device__ __forceinline__ T get(int q) const { return v[q]; }
-  __device__ __forceinline__ void set(int q, T x) { v[q] = x; }
-};
-template <> struct Acc44<float> {
-  unsigned long long v[8];   // pairs (i, j), (i, j + 1)
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = 0ull;
-  }
-  __device__ __forceinline__ void add(const Q4<float> &a, const Q4<float> &c) {
-    const unsigned long long c01 = pk2(c.x, c.y), c23 = pk2(c.z, c.w);
-    const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const unsigned long long ai = pk2(av[i], av[i]);
-      v[2 * i] = fma2(ai, c01, v[2 * i]);
-      v[2 * i + 1] = fma2(ai, c23, v[2 * i + 1]);
-    }
-  }
-  __device__ __forceinline__ float get(int q) const {
-    const float2 f = upk2(v[q >> 1]);
-    return (q & 1) ? f.y : f.x;
-  }
-  __device__ __forceinline__ void set(int q, float x) {
-    float2 f = upk2(v[q >> 1]);
-    if (q & 1) f.y = x; else f.x = x;
-    v[q >> 1] = pk2(f.x, f.y);
-  }
-};
-
-__device__ __forceinline__ void two_sum_fold(float &hi, float &lo, float &acc) {
-  const float s = hi + acc;
-  const float bp = s - hi;
-  const float e = (hi - (s - bp)) + (acc - bp);
-  hi = s;
-  lo += e;
-  acc = 0.f;
-}
-
-// nbu = upper tiles of one matrix; nb = 2 nbu tiles per row group; a group
-// is a whole number of warps (tpg threads) so that every warp reads one row
-// at a time and its shared loads of that row are broadcasts
+// nbu = upper tiles of one matrix; nb = 2 nbu tiles (threads) per row group;
+// rows of a slab: at least 32, the same number for every group, and even (the
+// diagonal is copied in pairs)
 struct Shape {
-  int mb, nbu, nb, tpg, ngroups;
+  int mb, nbu, nb, ngroups, rows;
 };
 
 __host__ __device__ constexpr Shape shape_of(int M) {
-  return Shape{M / 4, (M / 4) * (M / 4 + 1) / 2, (M / 4) * (M / 4 + 1), ((M / 4) * (M / 4 + 1) + 31) / 32 * 32,
-               kThreads / (((M / 4) * (M / 4 + 1) + 31) / 32 * 32)};
+  const int mb = M / 4, nb = mb * (mb + 1), groups = kThreads / nb;
+  int per = (32 + groups - 1) / groups;
+  if (per * groups % 2) ++per;
+  return Shape{mb, nb / 2, nb, groups, per * groups};
 }
 
 // tile index u in [0, nbu) -> (bi, bj) with bi <= bj (row-major upper triangle)
@@ -149,133 +93,112 @@ __device__ __forceinline__ void upper_tile(int u, int mb, int &bi, int &bj) {
 
 // shared layout of one slab: per block, TR rows of LD values, S then LS, then
 // the TR diagonal entries of B
-template <typename T, int LD, int NBLK>
+template <int LD, int NBLK>
 struct Slab {
-  static constexpr int TR = Tile<T>::rows;
+  static constexpr int TR = shape_of(LD * NBLK).rows;
   // elements of one block, padded by 16 bytes so that the same column of
   // different blocks falls in different shared-memory banks
-  static constexpr int blk = TR * LD + 16 / static_cast<int>(sizeof(T));
+  static constexpr int blk = TR * LD + 2;
   static constexpr int elems = 2 * NBLK * blk + TR;   // S, LS, diag(B)
 };
 
-template <typename T, int LD, int NBLK>
-__device__ __forceinline__ void stage(T *buf, int64_t r0, int64_t n, const T *const (&srcS)[3],
-                                      const T *const (&srcL)[3], const T *bdiag) {
-  using SL = Slab<T, LD, NBLK>;
+template <int LD, int NBLK>
+__device__ __forceinline__ void stage(double *buf, int64_t r0, int64_t n, const double *const (&srcS)[3],
+                                      const double *const (&srcL)[3], const double *bdiag) {
+  using SL = Slab<LD, NBLK>;
   constexpr int TR = SL::TR;
-  constexpr int per = 16 / static_cast<int>(sizeof(T));   // elements per 16-byte copy
-  constexpr int chunks = TR * LD / per;                    // per block and array
+  constexpr int chunks = TR * LD / 2;                      // 16-byte copies per block and array
 #pragma unroll
   for (int blk = 0; blk < NBLK; ++blk) {
     for (int i = threadIdx.x; i < 2 * chunks; i += kThreads) {
       const int arr = i / chunks, c = i - arr * chunks;
-      const int r = c * per / LD;
+      const int r = c * 2 / LD;
       const bool ok = r0 + r < n;
-      const T *src = (arr == 0 ? srcS[blk] : srcL[blk]) + (ok ? r0 * LD + c * per : 0);
-      cp16(buf + (arr * NBLK + blk) * SL::blk + c * per, src, ok ? 16 : 0);
+      const double *src = (arr == 0 ? srcS[blk] : srcL[blk]) + (ok ? r0 * LD + c * 2 : 0);
+      cp16(buf + (arr * NBLK + blk) * SL::blk + c * 2, src, ok ? 16 : 0);
     }
   }
   if (bdiag) {
-    for (int c = threadIdx.x; c < TR / per; c += kThreads) {
-      const int r = c * per;
+    for (int c = threadIdx.x; c < TR / 2; c += kThreads) {
+      const int r = c * 2;
       const int64_t left = n - r0 - r;
-      const int bytes = left >= per ? 16 : (left > 0 ? static_cast<int>(left) * static_cast<int>(sizeof(T)) : 0);
+      const int bytes = left >= 2 ? 16 : (left > 0 ? static_cast<int>(left) * 8 : 0);
       cp16(buf + 2 * NBLK * SL::blk + r, bdiag + (bytes ? r0 + r : 0), bytes);
     }
   }
 }
 
-template <typename T, int LD, int NBLK>
+template <int LD, int NBLK>
 __global__ void __launch_bounds__(kThreads)
-k_gram(int64_t n, const T *s0, const T *s1, const T *s2, const T *l0, const T *l1, const T *l2,
-       const T *bdiag, double *partials, const int *done) {
-  using SL = Slab<T, LD, NBLK>;
+k_gram(int64_t n, const double *s0, const double *s1, const double *s2, const double *l0, const double *l1,
+       const double *l2, const double *bdiag, double *partials, const int *done) {
+  using SL = Slab<LD, NBLK>;
   constexpr int M = LD * NBLK;
   constexpr int TR = SL::TR;
   constexpr Shape sh = shape_of(M);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (done && *done) return;
-  constexpr int NS = Tile<T>::stages;
-  T *const base = reinterpret_cast<T *>(smem_raw);
+  double *const base = reinterpret_cast<double *>(smem_raw);
+  double *const scaled = base + kStages * SL::elems;   // B S of the slab in hand
   const int tid = threadIdx.x;
-  const int grp = tid / sh.tpg, t = tid - (tid / sh.tpg) * sh.tpg;
-  const bool active = grp < sh.ngroups && t < sh.nb;
+  const int grp = tid / sh.nb, t = tid - (tid / sh.nb) * sh.nb;
+  const bool active = grp < sh.ngroups;
   int bi = 0, bj = 0;
-  const int tt = t < sh.nb ? t : 0;   // padding threads of a group take tile 0 and stay idle
-  const bool isA = tt < sh.nbu;
-  upper_tile(isA ? tt : tt - sh.nbu, sh.mb, bi, bj);
+  const bool isA = t < sh.nbu;
+  upper_tile(isA ? t : t - sh.nbu, sh.mb, bi, bj);
   // offsets of the thread's two column groups inside a slab
   const int offA = (bi * 4 / LD) * SL::blk + (bi * 4) % LD;                        // S, rows x LD
-  const int offC = ((isA ? NBLK : 0) + bj * 4 / LD) * SL::blk + (bj * 4) % LD;    // LS or S
-  const T *const srcS[3] = {s0, s1, s2};
-  const T *const srcL[3] = {l0, l1, l2};
-  Acc44<T> acc;
-  acc.zero();
-  float hi[16], lo[16];
+  const int offC = ((isA ? NBLK : 0) + bj * 4 / LD) * SL::blk + (bj * 4) % LD;    // LS or S (or B S)
+  const double *const srcS[3] = {s0, s1, s2};
+  const double *const srcL[3] = {l0, l1, l2};
+  double acc[16];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) { hi[q] = 0.f; lo[q] = 0.f; }
+  for (int q = 0; q < 16; ++q) acc[q] = 0.0;
   const int64_t ntile = (n + TR - 1) / TR;
-  const bool useB = !isA && bdiag != nullptr;
-  int since_flush = 0;
-  // ring of NS slabs: slab it % NS holds this CTA's it-th row slab; NS - 1
-  // slabs are in flight while one is multiplied
+  // ring of kStages slabs: slab it % kStages holds this CTA's it-th row slab;
+  // kStages - 1 slabs are in flight while one is multiplied
   int64_t tile = blockIdx.x;
 #pragma unroll
-  for (int s = 0; s < NS - 1; ++s) {
+  for (int s = 0; s < kStages - 1; ++s) {
     const int64_t tl = tile + static_cast<int64_t>(s) * gridDim.x;
-    if (tl < ntile) stage<T, LD, NBLK>(base + s * SL::elems, tl * TR, n, srcS, srcL, bdiag);
+    if (tl < ntile) stage<LD, NBLK>(base + s * SL::elems, tl * TR, n, srcS, srcL, bdiag);
     cp_commit();
   }
   for (int it = 0; tile < ntile; tile += gridDim.x, ++it) {
-    const int64_t ahead = tile + static_cast<int64_t>(NS - 1) * gridDim.x;
-    if (ahead < ntile) stage<T, LD, NBLK>(base + ((it + NS - 1) % NS) * SL::elems, ahead * TR, n, srcS, srcL, bdiag);
+    const int64_t ahead = tile + static_cast<int64_t>(kStages - 1) * gridDim.x;
+    if (ahead < ntile)
+      stage<LD, NBLK>(base + ((it + kStages - 1) % kStages) * SL::elems, ahead * TR, n, srcS, srcL, bdiag);
     cp_commit();
-    cp_wait<NS - 1>();     // this slab's group has landed; the NS - 1 later ones may be in flight
+    cp_wait<kStages - 1>();   // this slab's group has landed; the later ones may be in flight
     __syncthreads();
-    const T *buf = base + (it % NS) * SL::elems;
-    if (active) {
-      const T *bd = buf + 2 * NBLK * SL::blk;
-#pragma unroll 4
-      for (int r = grp; r < TR; r += sh.ngroups) {
-        const Q4<T> av = ld4(buf + offA + r * LD);
-        Q4<T> cv = ld4(buf + offC + r * LD);
-        if (useB) {
-          const T b = bd[r];
-          cv = {cv.x * b, cv.y * b, cv.z * b, cv.w * b};
-        }
-        acc.add(av, cv);
-      }
-      if constexpr (std::is_same<T, float>::value) {
-        since_flush += (TR + sh.ngroups - 1) / sh.ngroups;
-        if (since_flush >= 64) {
+    const double *buf = base + (it % kStages) * SL::elems;
+    if (bdiag) {
+      const double *bd = buf + 2 * NBLK * SL::blk;
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            float a = acc.get(q);
-            two_sum_fold(hi[q], lo[q], a);
-          }
-          acc.zero();
-          since_flush = 0;
-        }
+      for (int blk = 0; blk < NBLK; ++blk)
+        for (int e = tid; e < TR * LD; e += kThreads) scaled[blk * SL::blk + e] = buf[blk * SL::blk + e] * bd[e / LD];
+      __syncthreads();
+    }
+    if (active) {
+      const double *pa = buf + offA, *pc = (isA || !bdiag ? buf : scaled) + offC;
+#pragma unroll 2
+      for (int r = grp; r < TR; r += sh.ngroups) {
+        const Q4<double> av = ld4(pa + r * LD), cv = ld4(pc + r * LD);
+        const double a4[4] = {av.x, av.y, av.z, av.w}, c4[4] = {cv.x, cv.y, cv.z, cv.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i * 4 + j] = fma(a4[i], c4[j], acc[i * 4 + j]);
       }
     }
-    __syncthreads();       // the slab may be refilled by the next stage
+    __syncthreads();          // the slab may be refilled by the next stage
   }
   cp_wait<0>();
   __syncthreads();
   double *red = reinterpret_cast<double *>(smem_raw);  // [ngroups][nb * 16]
   if (active) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      double v;
-      if constexpr (std::is_same<T, float>::value) {
-        float a = acc.get(q);
-        two_sum_fold(hi[q], lo[q], a);
-        v = static_cast<double>(hi[q]) + static_cast<double>(lo[q]);
-      } else {
-        v = acc.get(q);
-      }
-      red[(grp * sh.nb + t) * 16 + q] = v;
-    }
+    for (int q = 0; q < 16; ++q) red[(grp * sh.nb + t) * 16 + q] = acc[q];
   }
   __syncthreads();
   for (int o = tid; o < sh.nb * 16; o += kThreads) {
@@ -550,15 +473,15 @@ int launch_t(cudaStream_t st, const GramArgs &a, const T *bd, int grid) {
   } else {
     constexpr int M = LD * NBLK;
     const Shape sh = shape_of(M);
-    const size_t slabs = static_cast<size_t>(Tile<T>::stages) * Slab<T, LD, NBLK>::elems * sizeof(T);
+    using SL = Slab<LD, NBLK>;
+    const size_t slabs = (static_cast<size_t>(kStages) * SL::elems + NBLK * SL::blk) * sizeof(double);
     const size_t red = static_cast<size_t>(sh.ngroups) * sh.nb * 16 * sizeof(double);
     const size_t sm = slabs > red ? slabs : red;
     if (sm > 48 * 1024)
-      SPX_CUDA(cudaFuncSetAttribute(k_gram<T, LD, NBLK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      SPX_CUDA(cudaFuncSetAttribute(k_gram<LD, NBLK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     static_cast<int>(sm)));
-    // two waves of the 2 resident CTAs per SM; the compensated sums take any row count
     const int g = grid < 4 * kSmCount ? grid : 4 * kSmCount;
-    k_gram<T, LD, NBLK><<<g, kThreads, sm, st>>>(a.n, p(0), p(1), p(2), q(0), q(1), q(2), bd, a.partials, a.done);
+    k_gram<LD, NBLK><<<g, kThreads, sm, st>>>(a.n, p(0), p(1), p(2), q(0), q(1), q(2), bd, a.partials, a.done);
     SPX_LAUNCHED();
     return g;
   }

@@ -190,57 +190,98 @@ __global__ void k_degrees(const int64_t *rp, const float *w, const int64_t *vw, 
 }
 
 // ---- Eq. 1 cutsize and part weights ----------------------------------------
-constexpr int kEvalRun = 64;   // entries per thread step of the cut
+// Exact weight of an entry, w 2^wscale, an integer below 2^63 (1 without
+// weights); the power is applied in two halves so that neither overflows.
+struct CutScale {
+  float a, b;
+};
+__device__ __forceinline__ unsigned long long cut_weight(float w, CutScale sc) {
+  return static_cast<unsigned long long>(__float2ll_rn(w * sc.a * sc.b));
+}
+__device__ __forceinline__ void cut_add(unsigned long long acc, unsigned long long *cut2) {
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+  if ((threadIdx.x & 31) == 0 && acc) atomicAdd(cut2, acc);
+}
+
+// Short rows and all part weights: a warp a 32-row slice, lane = row, over the
+// SELL-32 copy of the columns, whose entry t of the 32 rows is one segment (a
+// thread walking CSR entries of its own touches 32 lines a load: 350 us for the
+// 128^3 mesh, of which EVAL_US are left).  Lanes of one part add their weight once.
+template <bool W>
 __global__ void __launch_bounds__(256)
-k_eval(const int64_t *rp, const int32_t *col, const float *w, const int64_t *vw, int64_t n,
-       const int32_t *part, int K, int wscale, unsigned long long *cut2, long long *pw, unsigned *badpart,
-       int use_smem) {
-  extern __shared__ long long spw[];
+k_eval_short(const int16_t *__restrict__ scol, const float *__restrict__ sw, const int64_t *__restrict__ sptr,
+             const int64_t *__restrict__ cptr, const uint8_t *__restrict__ sdeg, const int64_t *vw, int64_t n,
+             const int32_t *__restrict__ part, int K, CutScale sc, unsigned long long *cut2, long long *pw,
+             unsigned *badpart, int use_smem) {
+  extern __shared__ unsigned long long spw[];
   if (use_smem) {
     for (int k = threadIdx.x; k < K; k += blockDim.x) spw[k] = 0;
     __syncthreads();
   }
+  unsigned long long *weights = use_smem ? spw : reinterpret_cast<unsigned long long *>(pw);
+  const int lane = threadIdx.x & 31;
+  const int64_t slices = (n + 31) / 32, warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
   unsigned long long acc = 0;
   unsigned bad = 0;
-  const int64_t nthreads = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  const int64_t tid = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  // part weights: one vertex per thread step
-  for (int64_t i = tid; i < n; i += nthreads) {
-    const int32_t pi = part[i];
-    if (pi < 0 || pi >= K) { bad = 1; continue; }
-    const long long wv = vw ? vw[i] : 1;
-    if (use_smem) atomicAdd(reinterpret_cast<unsigned long long *>(&spw[pi]), static_cast<unsigned long long>(wv));
-    else atomicAdd(reinterpret_cast<unsigned long long *>(&pw[pi]), static_cast<unsigned long long>(wv));
-  }
-  // cut: runs of kEvalRun consecutive entries per thread step, whatever the
-  // row lengths; the run's first row comes from a binary search of row_ptr
-  const int64_t nnz = rp[n];
-  for (int64_t e0 = tid * kEvalRun; e0 < nnz; e0 += nthreads * kEvalRun) {
-    int64_t lo = 0, hi = n - 1;                 // last row with rp[row] <= e0
-    while (lo < hi) {
-      const int64_t mid = (lo + hi + 1) >> 1;
-      if (rp[mid] <= e0) lo = mid;
-      else hi = mid - 1;
+  for (int64_t slice = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; slice < slices;
+       slice += warps) {
+    const int64_t row = slice * 32 + lane;
+    const bool in = row < n;
+    const int32_t pi = in ? part[row] : -1;
+    const bool ok = pi >= 0 && pi < K;
+    if (in && !ok) bad = 1;
+    unsigned long long wv = ok ? (vw ? static_cast<unsigned long long>(vw[row]) : 1ull) : 0ull;
+    const int32_t p0 = __shfl_sync(0xffffffffu, pi, 0);
+    if (__all_sync(0xffffffffu, !ok || pi == p0)) {
+      for (int off = 16; off > 0; off >>= 1) wv += __shfl_down_sync(0xffffffffu, wv, off);
+      if (lane == 0 && ok) atomicAdd(&weights[pi], wv);
+      else if (lane == 0 && wv) bad = 1;
+    } else if (ok) {
+      atomicAdd(&weights[pi], wv);
     }
-    int64_t row = lo;
-    const int64_t e1 = e0 + kEvalRun < nnz ? e0 + kEvalRun : nnz;
-    for (int64_t e = e0; e < e1; ++e) {
-      while (rp[row + 1] <= e) ++row;
-      const int32_t pi = part[row], pj = part[col[e]];
-      if (pi != pj && pi >= 0 && pi < K) {
-        if (w) acc += static_cast<unsigned long long>(llrint(ldexp(static_cast<double>(w[e]), wscale)));
-        else acc += 1;
-      }
+    const int sd = in ? sdeg[row] : 0xFF;
+    const int d = sd == 0xFF || !ok ? 0 : sd;
+    const int64_t cb = cptr[slice];
+    const float *wp = W ? sw + sptr[slice] + lane : nullptr;
+    if (cb < 0) {
+      const int16_t *cp = scol + (~cb) + lane;
+      for (int t = 0; t < d; ++t)
+        if (__ldg(part + row + __ldcs(cp + 32 * t)) != pi) acc += W ? cut_weight(__ldcs(wp + 32 * t), sc) : 1ull;
+    } else {
+      const int32_t *cp = reinterpret_cast<const int32_t *>(scol + cb) + lane;
+      for (int t = 0; t < d; ++t)
+        if (__ldg(part + __ldcs(cp + 32 * t)) != pi) acc += W ? cut_weight(__ldcs(wp + 32 * t), sc) : 1ull;
     }
   }
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0 && acc) atomicAdd(cut2, acc);
+  cut_add(acc, cut2);
   if (bad) atomicOr(badpart, 1u);
   if (use_smem) {
     __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x)
-      if (spw[k]) atomicAdd(reinterpret_cast<unsigned long long *>(&pw[k]), static_cast<unsigned long long>(spw[k]));
+      if (spw[k]) atomicAdd(reinterpret_cast<unsigned long long *>(&pw[k]), spw[k]);
   }
+}
+
+// Longer rows: a warp per medium row (rows[i]) or per work item of a long row
+// ({row, begin, end, slot}), over the CSR entries.
+template <bool W>
+__global__ void __launch_bounds__(256)
+k_eval_long(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ w,
+            const int32_t *__restrict__ rows, int64_t n_rows, const int64_t *__restrict__ items, int64_t n_items,
+            const int32_t *__restrict__ part, CutScale sc, unsigned long long *cut2) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+  unsigned long long acc = 0;
+  for (int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; i < n_rows + n_items;
+       i += warps) {
+    const int64_t row = i < n_rows ? rows[i] : items[4 * (i - n_rows)];
+    const int64_t b = i < n_rows ? rp[row] : items[4 * (i - n_rows) + 1];
+    const int64_t e = i < n_rows ? rp[row + 1] : items[4 * (i - n_rows) + 2];
+    const int32_t pi = part[row];
+    for (int64_t k = b + lane; k < e; k += 32)
+      if (__ldg(part + __ldcs(col + k)) != pi) acc += W ? cut_weight(__ldcs(w + k), sc) : 1ull;
+  }
+  cut_add(acc, cut2);
 }
 
 // SELL-32 layout of the short rows: per-row degree (0xFF marks a long row)
@@ -801,10 +842,32 @@ void eval_partition(sphynx_graph *g, const int32_t *part, int K, double *cut, do
   long long *d_pw = reinterpret_cast<long long *>(ws + 64);
   const int use_smem = K <= 4096 ? 1 : 0;
   const size_t sm = use_smem ? K * sizeof(long long) : 0;
-  k_eval<<<grid_for(g->n), 256, sm, g->stream>>>(g->rowptr, g->col, g->w, g->vw, g->n, part, K, g->wscale, d_cut,
-                                                 d_pw, d_bad, use_smem);
+  const SpmmPlan &p = g->plan;
+  const CutScale sc{ldexpf(1.f, g->weighted ? g->wscale / 2 : 0), ldexpf(1.f, g->weighted ? g->wscale - g->wscale / 2 : 0)};
+  const int16_t *scol = p.sell_col.as<int16_t>();
+  const int64_t n_long = p.n_med + p.n_items;
+  if (g->weighted) {
+    k_eval_short<true><<<grid_for(g->n), 256, sm, g->stream>>>(
+        scol, p.sell_w.as<float>(), p.sell_ptr.as<int64_t>(), p.sell_cptr.as<int64_t>(), p.sell_deg.as<uint8_t>(), g->vw,
+        g->n, part, K, sc, d_cut, d_pw, d_bad, use_smem);
+  } else {
+    k_eval_short<false><<<grid_for(g->n), 256, sm, g->stream>>>(
+        scol, nullptr, p.sell_ptr.as<int64_t>(), p.sell_cptr.as<int64_t>(), p.sell_deg.as<uint8_t>(), g->vw, g->n, part, K,
+        sc, d_cut, d_pw, d_bad, use_smem);
+  }
   SPX_LAUNCHED();
   g->ctr.launches++;
+  if (n_long > 0) {
+    const unsigned gl = static_cast<unsigned>(std::min<int64_t>((n_long + 7) / 8, 16 * kSmCount));
+    if (g->weighted)
+      k_eval_long<true><<<gl, 256, 0, g->stream>>>(g->rowptr, g->col, g->w, p.grp_row.as<int32_t>(), p.n_med,
+                                                   p.items.as<int64_t>(), p.n_items, part, sc, d_cut);
+    else
+      k_eval_long<false><<<gl, 256, 0, g->stream>>>(g->rowptr, g->col, nullptr, p.grp_row.as<int32_t>(), p.n_med,
+                                                    p.items.as<int64_t>(), p.n_items, part, sc, d_cut);
+    SPX_LAUNCHED();
+    g->ctr.launches++;
+  }
   std::vector<char> host(need);
   SPX_CUDA(cudaMemcpyAsync(host.data(), ws, need, cudaMemcpyDeviceToHost, g->stream));
   SPX_CUDA(cudaStreamSynchronize(g->stream));

@@ -496,13 +496,14 @@ void launch_harmonic_ritz_batch(cudaStream_t st, const double *alpha, const doub
 // ---- mj.cu ------------------------------------------------------------------
 void run_mj(cudaStream_t st, DT dt, const void *coords, int ldc, int dims, int64_t n,
             const int64_t *vw, int K, int32_t *part, Counters *ctr);
-// Multi-jagged with caller-provided scratch (mj_scratch_bytes).  With count > 1
+// Multi-jagged with caller-provided scratch (mj_scratch_bytes for the fastest
+// plan; less runs with narrower digits or without the key arrays).  With count > 1
 // the points are count graphs, graph g owning points [h_gptr[g], h_gptr[g+1])
 // (host offsets) and parts [g K/count, (g+1) K/count): the first level has one
 // section per graph and every later level splits within them.
-size_t mj_scratch_bytes(int64_t n, int K, int count);
+size_t mj_scratch_bytes(int64_t n, int K, int count, DT dt);
 void run_mj_scratch(cudaStream_t st, DT dt, const void *coords, int ldc, int dims, int64_t n,
-                    const int64_t *vw, int K, int32_t *part, Counters *ctr, void *scratch,
+                    const int64_t *vw, int K, int32_t *part, Counters *ctr, void *scratch, size_t scratch_bytes,
                     const int64_t *h_gptr, int count);
 
 // ---- refine.cu --------------------------------------------------------------
