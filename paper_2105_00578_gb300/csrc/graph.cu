@@ -10,6 +10,7 @@
 #include <cstdarg>
 #include <cstring>
 #include <memory>
+#include <mutex>
 
 namespace sphynx {
 
@@ -49,6 +50,52 @@ void DevBuf::alloc(size_t nbytes) {
     fail(SPHYNX_ERR_OOM, "cudaMalloc of %zu bytes failed: %s", nbytes, cudaGetErrorString(e));
   }
   bytes = nbytes;
+}
+
+namespace {
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pool[kMaxDevices] = {};   // NULL until first used
+
+// the library's pool of the current device (NULL: none can be made)
+cudaMemPool_t scratch_pool() {
+  int dev = 0;
+  SPX_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kScratchKeep;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+    g_pool[dev] = pool;
+  }
+  return g_pool[dev];
+}
+}  // namespace
+
+Scratch::Scratch(size_t bytes, cudaStream_t stream) : st(stream) {
+  const cudaMemPool_t pool = scratch_pool();
+  const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st) : cudaMallocAsync(&p, bytes, st);
+  if (e != cudaSuccess) {
+    p = nullptr;
+    cudaGetLastError();
+    fail(e == cudaErrorMemoryAllocation ? SPHYNX_ERR_OOM : SPHYNX_ERR_CUDA, "scratch of %zu bytes: %s", bytes,
+         cudaGetErrorString(e));
+  }
+}
+
+void scratch_trim(int device) {
+  if (device < 0 || device >= kMaxDevices) return;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (g_pool[device] && cudaMemPoolTrimTo(g_pool[device], 0) != cudaSuccess) cudaGetLastError();
 }
 
 void DevBuf::release() {
@@ -1037,7 +1084,9 @@ void sphynx_destroy(sphynx_handle g) {
   if (g->amg) amg_free(g->amg);
   for (auto e : g->ctr.ev_pool) cudaEventDestroy(e);
   if (g->host_flag) cudaFreeHost(g->host_flag);
+  const int device = g->device;
   delete g;
+  scratch_trim(device);
 }
 
 int sphynx_get_info(sphynx_handle g, sphynx_graph_info *info) {

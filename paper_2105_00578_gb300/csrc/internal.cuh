@@ -69,6 +69,22 @@ struct DevBuf {
   template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
+// Stream-ordered scratch of one call, from the library's own memory pool of the
+// current device.  The pool keeps up to kScratchKeep bytes between calls (the
+// default pool returns everything at each synchronisation, so that a call paid
+// about 200 us for mapping a few MB again) and gives them back when a handle is
+// destroyed; the driver orders its reuse across streams and threads.
+constexpr size_t kScratchKeep = size_t(64) << 20;
+struct Scratch {
+  void *p = nullptr;
+  cudaStream_t st;
+  Scratch(size_t bytes, cudaStream_t stream);   // throws OOM
+  ~Scratch() { if (p) cudaFreeAsync(p, st); }
+  Scratch(const Scratch &) = delete;
+  Scratch &operator=(const Scratch &) = delete;
+};
+void scratch_trim(int device);
+
 // Block element types used by the kernels.
 enum class DT { F64 = SPHYNX_DT_F64, F32 = SPHYNX_DT_F32, BF16 = SPHYNX_DT_BF16 };
 inline size_t dt_size(DT d) { return d == DT::F64 ? 8 : (d == DT::F32 ? 4 : 2); }

@@ -696,16 +696,9 @@ void run_mj_scratch(cudaStream_t st, DT dt, const void *coords, int ldc, int dim
 
 void run_mj(cudaStream_t st, DT dt, const void *coords, int ldc, int dims, int64_t n, const int64_t *vw, int K,
             int32_t *part, Counters *ctr) {
-  void *scratch = nullptr;
   const size_t bytes = mj_scratch_bytes(n, K, 1, dt);
-  SPX_CUDA(cudaMallocAsync(&scratch, bytes, st));
-  try {
-    run_mj_scratch(st, dt, coords, ldc, dims, n, vw, K, part, ctr, scratch, bytes, nullptr, 1);
-  } catch (...) {
-    cudaFreeAsync(scratch, st);
-    throw;
-  }
-  SPX_CUDA(cudaFreeAsync(scratch, st));
+  Scratch scratch(bytes, st);
+  run_mj_scratch(st, dt, coords, ldc, dims, n, vw, K, part, ctr, scratch.p, bytes, nullptr, 1);
 }
 
 }  // namespace sphynx
