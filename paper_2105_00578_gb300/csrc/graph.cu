@@ -336,16 +336,18 @@ k_eval_long(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, con
 // Per slice of 32 rows: the largest short-row degree, the number of
 // short-row entries, and whether every such entry lies within 32767 of its row
 // (then the slice stores 16-bit offsets).  Blocks are whole warps.
-__global__ void k_sell_deg(const int64_t *rp, const int32_t *col, int64_t n, uint8_t *sdeg, int *smax, int *ssum,
-                           int *sfit) {
-  const int64_t row = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+// Slot i is row sell_slot_row(i).
+__global__ void k_sell_deg(const int64_t *rp, const int32_t *col, int64_t n, const uint16_t *order, uint8_t *sdeg,
+                           int *smax, int *ssum, int *sfit) {
+  const int64_t slot = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   int d = 0, sd = 0xFF;
   bool fit = true;
-  if (row < n) {
+  if (slot < n) {
+    const int64_t row = sell_slot_row(order, slot);
     const int64_t dd = rp[row + 1] - rp[row];
     d = dd > (1 << 30) ? (1 << 30) : static_cast<int>(dd);
     sd = d > kShortDeg ? 0xFF : d;
-    sdeg[row] = static_cast<uint8_t>(sd);
+    sdeg[slot] = static_cast<uint8_t>(sd);
     if (sd != 0xFF) {
       const int64_t b = rp[row];
       for (int t = 0; t < d; ++t) {
@@ -361,20 +363,46 @@ __global__ void k_sell_deg(const int64_t *rp, const int32_t *col, int64_t n, uin
     s += __shfl_down_sync(0xffffffffu, s, off);
   }
   fit = __all_sync(0xffffffffu, fit);
-  if ((threadIdx.x & 31) == 0 && row < n) {
-    smax[row >> 5] = m;
-    ssum[row >> 5] = s;
-    sfit[row >> 5] = fit ? 1 : 0;
+  if ((threadIdx.x & 31) == 0 && slot < n) {
+    smax[slot >> 5] = m;
+    ssum[slot >> 5] = s;
+    sfit[slot >> 5] = fit ? 1 : 0;
   }
 }
 
-__global__ void k_sell_fill(const int64_t *rp, const int32_t *col, const float *w, int64_t n, const uint8_t *sdeg,
-                            const int64_t *sptr, const int64_t *cptr, int16_t *scol, float *sw) {
-  const int64_t row = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (row >= n) return;
-  const int d = sdeg[row];
+// order[i] of each 1024-row window: its rows by decreasing degree (at most
+// kShortDeg), lowest row first on ties; one CTA of 1024 threads per window
+__global__ void __launch_bounds__(1024) k_sell_order(const int64_t *rp, int64_t n, uint16_t *order) {
+  __shared__ int cnt[32][kShortDeg + 1];   // rows of each warp per degree, then their first slots
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t row = static_cast<int64_t>(blockIdx.x) * 1024 + tid;
+  const int d = row < n ? static_cast<int>(rp[row + 1] - rp[row]) : -1;
+  for (int k = tid; k < 32 * (kShortDeg + 1); k += 1024) cnt[k / (kShortDeg + 1)][k % (kShortDeg + 1)] = 0;
+  __syncthreads();
+  const unsigned same = __match_any_sync(0xffffffffu, d);
+  const int rank = __popc(same & ((1u << lane) - 1u));
+  if (d >= 0 && rank == 0) cnt[warp][d] = __popc(same);
+  __syncthreads();
+  if (tid == 0) {
+    int at = 0;
+    for (int k = kShortDeg; k >= 0; --k)
+      for (int w = 0; w < 32; ++w) {
+        const int c = cnt[w][k];
+        cnt[w][k] = at;
+        at += c;
+      }
+  }
+  __syncthreads();
+  if (d >= 0) order[static_cast<int64_t>(blockIdx.x) * 1024 + cnt[warp][d] + rank] = static_cast<uint16_t>(tid);
+}
+
+__global__ void k_sell_fill(const int64_t *rp, const int32_t *col, const float *w, int64_t n, const uint16_t *order,
+                            const uint8_t *sdeg, const int64_t *sptr, const int64_t *cptr, int16_t *scol, float *sw) {
+  const int64_t slot = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (slot >= n) return;
+  const int d = sdeg[slot];
   if (d == 0xFF) return;
-  const int64_t slice = row >> 5, lane = row & 31, src = rp[row];
+  const int64_t row = sell_slot_row(order, slot), slice = slot >> 5, lane = slot & 31, src = rp[row];
   const int64_t cp = cptr[slice];
   if (cp < 0) {
     int16_t *c16 = scol + (~cp) + lane;
@@ -685,100 +713,166 @@ void build_plan(sphynx_graph *g, const int64_t *host_rowptr, int med_max) {
   }
 }
 
+// per slice: the largest short degree, the short entries, 16-bit offsets or not
+struct SliceStats {
+  std::vector<int> v;
+  int64_t slices;
+  const int *max() const { return v.data(); }
+  const int *sum() const { return v.data() + slices; }
+  const int *fit() const { return v.data() + 2 * slices; }
+  int64_t padded() const {
+    int64_t e = 0;
+    for (int64_t s = 0; s < slices; ++s) e += 32 * static_cast<int64_t>(max()[s]);
+    return e;
+  }
+};
+
+SliceStats slice_stats(sphynx_graph *g, const uint16_t *order, uint8_t *deg) {
+  SliceStats st;
+  st.slices = (g->n + 31) / 32;
+  st.v.resize(static_cast<size_t>(st.slices) * 3);
+  DevBuf d;
+  d.alloc(st.v.size() * sizeof(int));
+  k_sell_deg<<<static_cast<unsigned>((g->n + 255) / 256), 256, 0, g->stream>>>(
+      g->rowptr, g->col, g->n, order, deg, d.as<int>(), d.as<int>() + st.slices, d.as<int>() + 2 * st.slices);
+  SPX_LAUNCHED();
+  SPX_CUDA(cudaMemcpyAsync(st.v.data(), d.p, st.v.size() * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  SPX_CUDA(cudaStreamSynchronize(g->stream));
+  return st;
+}
+
+struct SliceLayout {
+  std::vector<int64_t> ptr, cptr;   // as SpmmPlan::sell_ptr and sell_cptr
+  int64_t narrow = 0;
+  double idx_bytes = 0, entries = 0;
+};
+
+// offsets of the slices, and their columns and weights into col_out / w_out
+SliceLayout fill_slices(sphynx_graph *g, const SliceStats &st, const uint16_t *order, const uint8_t *deg, DevBuf &ptr,
+                        DevBuf &cptr, DevBuf &col_out, DevBuf &w_out) {
+  SliceLayout l;
+  const int64_t slices = st.slices;
+  l.ptr.assign(static_cast<size_t>(slices) + 1, 0);
+  l.cptr.assign(static_cast<size_t>(slices), 0);
+  int64_t units = 0;
+  for (int64_t s = 0; s < slices; ++s) {
+    const int64_t m = st.max()[s];
+    l.ptr[s + 1] = l.ptr[s] + 32 * m;
+    if (st.fit()[s]) {
+      l.cptr[s] = ~units;
+      units += 32 * m;
+      ++l.narrow;
+      l.idx_bytes += 2.0 * st.sum()[s];
+    } else {
+      units = (units + 63) & ~static_cast<int64_t>(63);   // 128-byte aligned rows of 32 indices
+      l.cptr[s] = units;
+      units += 64 * m;
+      l.idx_bytes += 4.0 * st.sum()[s];
+    }
+    l.entries += st.sum()[s];
+  }
+  ptr.alloc(l.ptr.size() * sizeof(int64_t));
+  cptr.alloc(l.cptr.size() * sizeof(int64_t) + 8);
+  SPX_CUDA(cudaMemcpyAsync(ptr.p, l.ptr.data(), l.ptr.size() * sizeof(int64_t), cudaMemcpyHostToDevice, g->stream));
+  SPX_CUDA(cudaMemcpyAsync(cptr.p, l.cptr.data(), l.cptr.size() * sizeof(int64_t), cudaMemcpyHostToDevice, g->stream));
+  col_out.alloc(static_cast<size_t>(units > 0 ? units : 1) * sizeof(int16_t));
+  if (g->weighted) w_out.alloc(static_cast<size_t>(l.ptr[slices] > 0 ? l.ptr[slices] : 1) * sizeof(float));
+  k_sell_fill<<<static_cast<unsigned>((g->n + 255) / 256), 256, 0, g->stream>>>(
+      g->rowptr, g->col, g->w, g->n, order, deg, ptr.as<int64_t>(), cptr.as<int64_t>(), col_out.as<int16_t>(),
+      w_out.as<float>());
+  SPX_LAUNCHED();
+  SPX_CUDA(cudaStreamSynchronize(g->stream));   // `l` may go out of scope
+  return l;
+}
+
+// The degree-ordered copy for double products, where it makes the slices a
+// sixth shorter: the FP64 pipe takes 64 cycles an instruction of a warp, which
+// runs to the longest row of its slice, and a geometric graph's longest of 32
+// rows has nearly twice the mean.  300,000-vertex geometric graph, 4 columns:
+// chain step 61 -> 39 us.  Float products of that graph take 21 us in natural
+// order and 24 in this one.  Only for graphs of short rows without
+// shared-pattern slices (meshes: their rows are equally long already).
+void build_degree_slices(sphynx_graph *g, int64_t natural_padded) {
+  SpmmPlan &p = g->plan;
+  p.deg_row.release();
+  if (p.pat_slices > 0 || g->max_degree > kShortDeg || g->n <= 32) return;
+  const int64_t n = g->n;
+  p.deg_row.alloc(static_cast<size_t>(n) * sizeof(uint16_t));
+  p.deg_deg.alloc(static_cast<size_t>(n));
+  k_sell_order<<<static_cast<unsigned>((n + 1023) / 1024), 1024, 0, g->stream>>>(g->rowptr, n, p.deg_row.as<uint16_t>());
+  SPX_LAUNCHED();
+  const SliceStats st = slice_stats(g, p.deg_row.as<uint16_t>(), p.deg_deg.as<uint8_t>());
+  if (6 * st.padded() > 5 * natural_padded) {
+    p.deg_row.release();
+    p.deg_deg.release();
+    return;
+  }
+  p.deg_narrow = fill_slices(g, st, p.deg_row.as<uint16_t>(), p.deg_deg.as<uint8_t>(), p.deg_ptr, p.deg_cptr, p.deg_col,
+                             p.deg_w).narrow;
+}
+
 void build_sell(sphynx_graph *g) {
   SpmmPlan &p = g->plan;
   const int64_t n = g->n, slices = (n + 31) / 32;
   p.sell_deg.alloc(static_cast<size_t>(n));
-  DevBuf sstat;
-  sstat.alloc(static_cast<size_t>(slices) * 3 * sizeof(int));
-  int *smax = sstat.as<int>(), *ssum = smax + slices, *sfit = ssum + slices;
-  const unsigned blocks = static_cast<unsigned>((n + 255) / 256);
-  k_sell_deg<<<blocks, 256, 0, g->stream>>>(g->rowptr, g->col, n, p.sell_deg.as<uint8_t>(), smax, ssum, sfit);
-  SPX_LAUNCHED();
-  std::vector<int> hstat(static_cast<size_t>(slices) * 3);
-  SPX_CUDA(cudaMemcpyAsync(hstat.data(), sstat.p, hstat.size() * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
-  SPX_CUDA(cudaStreamSynchronize(g->stream));
-  const int *hmax = hstat.data(), *hsum = hmax + slices, *hfit = hsum + slices;
-  std::vector<int64_t> hptr(static_cast<size_t>(slices) + 1, 0), hcptr(static_cast<size_t>(slices), 0);
-  int64_t units = 0, narrow = 0;
-  double idx_bytes = 0, entries = 0;
-  for (int64_t s = 0; s < slices; ++s) {
-    hptr[s + 1] = hptr[s] + 32 * static_cast<int64_t>(hmax[s]);
-    if (hfit[s]) {
-      hcptr[s] = ~units;
-      units += 32 * static_cast<int64_t>(hmax[s]);
-      ++narrow;
-      idx_bytes += 2.0 * hsum[s];
-    } else {
-      units = (units + 63) & ~static_cast<int64_t>(63);   // 128-byte aligned rows of 32 indices
-      hcptr[s] = units;
-      units += 64 * static_cast<int64_t>(hmax[s]);
-      idx_bytes += 4.0 * hsum[s];
-    }
-    entries += hsum[s];
-  }
-  p.sell_entries = hptr[slices];
-  p.sell_narrow = narrow;
-  p.short_entries = entries;
+  const SliceStats st = slice_stats(g, nullptr, p.sell_deg.as<uint8_t>());
+  const int *hsum = st.sum();
+  const SliceLayout lay = fill_slices(g, st, nullptr, p.sell_deg.as<uint8_t>(), p.sell_ptr, p.sell_cptr, p.sell_col,
+                                      p.sell_w);
+  const std::vector<int64_t> &hcptr = lay.cptr;
+  p.sell_entries = lay.ptr[slices];
+  p.sell_narrow = lay.narrow;
+  p.short_entries = lay.entries;
   // indices of the real entries, the degree bytes and one slice offset per slice
   // (plus the weights and their offsets on weighted graphs)
-  p.sell_bytes = idx_bytes + static_cast<double>(n) + 8.0 * static_cast<double>(slices) +
-                 (g->weighted ? 4.0 * entries + 8.0 * static_cast<double>(slices) : 0.0);
-  p.sell_ptr.alloc(hptr.size() * sizeof(int64_t));
-  p.sell_cptr.alloc(hcptr.size() * sizeof(int64_t) + 8);
-  SPX_CUDA(cudaMemcpyAsync(p.sell_ptr.p, hptr.data(), hptr.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
-                           g->stream));
-  SPX_CUDA(cudaMemcpyAsync(p.sell_cptr.p, hcptr.data(), hcptr.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
-                           g->stream));
-  p.sell_col.alloc(static_cast<size_t>(units > 0 ? units : 1) * sizeof(int16_t));
-  if (g->weighted) p.sell_w.alloc(static_cast<size_t>(p.sell_entries > 0 ? p.sell_entries : 1) * sizeof(float));
-  k_sell_fill<<<blocks, 256, 0, g->stream>>>(g->rowptr, g->col, g->w, n, p.sell_deg.as<uint8_t>(),
-                                             p.sell_ptr.as<int64_t>(), p.sell_cptr.as<int64_t>(),
-                                             p.sell_col.as<int16_t>(), p.sell_w.as<float>());
-  SPX_LAUNCHED();
+  p.sell_bytes = lay.idx_bytes + static_cast<double>(n) + 8.0 * static_cast<double>(slices) +
+                 (g->weighted ? 4.0 * lay.entries + 8.0 * static_cast<double>(slices) : 0.0);
   // the shared-pattern variant (unweighted graphs with at least one such slice)
+  std::vector<int> hnu;
+  int64_t npat = 0;
+  const unsigned wblocks = static_cast<unsigned>((slices * 32 + 255) / 256);
+  if (!g->weighted && slices > 0) {
+    DevBuf nub;
+    nub.alloc(static_cast<size_t>(slices) * sizeof(int));
+    k_sell_pattern<<<wblocks, 256, 0, g->stream>>>(g->rowptr, g->col, n, p.sell_deg.as<uint8_t>(), nub.as<int>());
+    SPX_LAUNCHED();
+    hnu.resize(static_cast<size_t>(slices));
+    SPX_CUDA(cudaMemcpyAsync(hnu.data(), nub.p, hnu.size() * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+    SPX_CUDA(cudaStreamSynchronize(g->stream));
+    for (int64_t s = 0; s < slices; ++s) npat += hnu[s] >= 0 ? 1 : 0;
+  }
   p.pat_slices = 0;
   p.pat_all = false;
   p.pat_cptr.release();
   p.pat_col.release();
-  if (!g->weighted && slices > 0) {
-    DevBuf nub;
-    nub.alloc(static_cast<size_t>(slices) * sizeof(int));
-    const unsigned wblocks = static_cast<unsigned>((slices * 32 + 255) / 256);
-    k_sell_pattern<<<wblocks, 256, 0, g->stream>>>(g->rowptr, g->col, n, p.sell_deg.as<uint8_t>(), nub.as<int>());
-    SPX_LAUNCHED();
-    std::vector<int> hnu(static_cast<size_t>(slices));
-    SPX_CUDA(cudaMemcpyAsync(hnu.data(), nub.p, hnu.size() * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
-    SPX_CUDA(cudaStreamSynchronize(g->stream));
+  if (npat > 0) {
     std::vector<int64_t> pc(static_cast<size_t>(slices));
-    int64_t punits = 0, npat = 0;
+    int64_t punits = 0;
     double pbytes = 0;
     for (int64_t s = 0; s < slices; ++s) {
       if (hnu[s] >= 0) {
         pc[s] = kPatternTag | punits;
         punits += 96;   // 64 bytes of offsets, 128 bytes of masks
         pbytes += 192.0;
-        ++npat;
       } else {
         pc[s] = hcptr[s];
         const double rows = static_cast<double>(std::min<int64_t>(32, n - 32 * s));
         pbytes += (hcptr[s] < 0 ? 2.0 : 4.0) * hsum[s] + rows;
       }
     }
-    if (npat > 0) {
-      p.pat_slices = npat;
-      p.pat_all = npat == slices;
-      p.pat_bytes = pbytes + 8.0 * static_cast<double>(slices);
-      p.pat_cptr.alloc(pc.size() * sizeof(int64_t));
-      p.pat_col.alloc(static_cast<size_t>(punits) * sizeof(int16_t));
-      SPX_CUDA(cudaMemcpyAsync(p.pat_cptr.p, pc.data(), pc.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
-                               g->stream));
-      k_pat_fill<<<wblocks, 256, 0, g->stream>>>(g->rowptr, g->col, n, p.sell_deg.as<uint8_t>(),
-                                                 p.pat_cptr.as<int64_t>(), p.pat_col.as<int16_t>());
-      SPX_LAUNCHED();
-    }
+    p.pat_slices = npat;
+    p.pat_all = npat == slices;
+    p.pat_bytes = pbytes + 8.0 * static_cast<double>(slices);
+    p.pat_cptr.alloc(pc.size() * sizeof(int64_t));
+    p.pat_col.alloc(static_cast<size_t>(punits) * sizeof(int16_t));
+    SPX_CUDA(cudaMemcpyAsync(p.pat_cptr.p, pc.data(), pc.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
+                             g->stream));
+    k_pat_fill<<<wblocks, 256, 0, g->stream>>>(g->rowptr, g->col, n, p.sell_deg.as<uint8_t>(),
+                                               p.pat_cptr.as<int64_t>(), p.pat_col.as<int16_t>());
+    SPX_LAUNCHED();
   }
   SPX_CUDA(cudaStreamSynchronize(g->stream));
+  build_degree_slices(g, st.padded());
 }
 
 // Staged blocks, for graphs whose every slice is a shared-pattern slice and
@@ -895,12 +989,12 @@ void eval_partition(sphynx_graph *g, const int32_t *part, int K, double *cut, do
   const int64_t n_long = p.n_med + p.n_items;
   if (g->weighted) {
     k_eval_short<true><<<grid_for(g->n), 256, sm, g->stream>>>(
-        scol, p.sell_w.as<float>(), p.sell_ptr.as<int64_t>(), p.sell_cptr.as<int64_t>(), p.sell_deg.as<uint8_t>(), g->vw,
-        g->n, part, K, sc, d_cut, d_pw, d_bad, use_smem);
+        scol, p.sell_w.as<float>(), p.sell_ptr.as<int64_t>(), p.sell_cptr.as<int64_t>(), p.sell_deg.as<uint8_t>(),
+        g->vw, g->n, part, K, sc, d_cut, d_pw, d_bad, use_smem);
   } else {
     k_eval_short<false><<<grid_for(g->n), 256, sm, g->stream>>>(
-        scol, nullptr, p.sell_ptr.as<int64_t>(), p.sell_cptr.as<int64_t>(), p.sell_deg.as<uint8_t>(), g->vw, g->n, part, K,
-        sc, d_cut, d_pw, d_bad, use_smem);
+        scol, nullptr, p.sell_ptr.as<int64_t>(), p.sell_cptr.as<int64_t>(), p.sell_deg.as<uint8_t>(),
+        g->vw, g->n, part, K, sc, d_cut, d_pw, d_bad, use_smem);
   }
   SPX_LAUNCHED();
   g->ctr.launches++;

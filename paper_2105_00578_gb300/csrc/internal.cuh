@@ -123,6 +123,11 @@ constexpr int kBlkThreads = 128;                 // threads of a staged block, o
 constexpr size_t kBlkSmemMax = 200 * 1024;       // shared memory a staged block may take
 constexpr int kSellLsCount = 5;      // slice strides 1, 2, 4, 8, 16 the autotuner times
 
+// the row of a SELL-32 slot (order: SpmmPlan::deg_row, NULL for natural order)
+__device__ __forceinline__ int64_t sell_slot_row(const uint16_t *order, int64_t slot) {
+  return order ? (slot & ~int64_t{1023}) + order[slot] : slot;
+}
+
 struct SpmmTuning {
   int variant;
   float us[kSpmmVariants];           // measured time of each schedule (1e30: not available)
@@ -157,6 +162,12 @@ struct SpmmPlan {
   DevBuf sell_col;                   // 16-bit units [sum of block sizes]
   DevBuf sell_w;                     // float [sell_entries] (weighted graphs)
   DevBuf sell_deg;                   // uint8 [n]: degree, or 0xFF for a long row
+  // The same layout with the rows of each 1024-row window by decreasing degree,
+  // so that a slice's rows are equally long: slot i (lane i & 31 of slice i >> 5)
+  // is row (i & ~1023) + deg_row[i].  Double products read it where it is built.
+  DevBuf deg_row;                    // uint16 [n], or none
+  DevBuf deg_ptr, deg_cptr, deg_col, deg_w, deg_deg;   // as sell_*, by slot
+  int64_t deg_narrow = 0;
   // Shared-pattern slices (unweighted graphs): a slice whose 32 rows' short-row
   // offsets col - row take at most 31 distinct values, all within 16 bits,
   // stores that sorted union U once (32 int16, zero padded: 64 bytes) and one

@@ -214,7 +214,11 @@ void spmm(sphynx_graph *g, const SpmmArgs &a) {
   }
 
   // schedule: forced, or the one the autotuner chose for this graph at create
-  g->plan.variant = g->plan.forced >= 0 ? g->plan.forced : g->plan.tuned_variant;
+  // from a float product.  Double products take the degree-ordered slices
+  // wherever those exist (300,000-vertex geometric graph, 4 columns, a chain
+  // step: 59.5 us in the CSR schedule, 39.2 in these).
+  g->plan.variant = g->plan.forced >= 0 ? g->plan.forced
+                    : a.tin == DT::F64 && g->plan.deg_row.p ? static_cast<int>(kSell32) : g->plan.tuned_variant;
 
   // algorithmic bytes: the graph in the layout the schedule reads (CSR row
   // pointers and indices, or the SELL-32 slices plus the long rows' CSR

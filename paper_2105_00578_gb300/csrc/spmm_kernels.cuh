@@ -816,10 +816,13 @@ template <int LAP, typename TI, typename TT, int BP, bool W, int MODE, int KIND>
 __device__ __forceinline__ void sell_slice(const LapView &L, const SpmmDev &a, const int16_t *__restrict__ scol,
                                            const float *__restrict__ sw, const int64_t *__restrict__ sptr,
                                            const int64_t *__restrict__ cptr, const uint8_t *__restrict__ sdeg,
-                                           const int16_t *__restrict__ pcol, int64_t slice, int lane) {
+                                           const int16_t *__restrict__ pcol, const uint16_t *__restrict__ srow,
+                                           int64_t slice, int lane) {
   using TA = typename AccOf<TI>::T;
   if (slice * 32 >= L.n) return;  // uniform per warp
-  const int64_t row = slice * 32 + lane;
+  const int64_t slot = slice * 32 + lane;
+  // degree-ordered slices: double products only
+  const int64_t row = std::is_same<TI, double>::value && KIND < 2 && srow && slot < L.n ? sell_slot_row(srow, slot) : slot;
   const int64_t cbase = __ldg(cptr + slice);
   const TI *__restrict__ x = static_cast<const TI *>(a.x);
   RowAcc<TI, BP> acc;
@@ -841,8 +844,8 @@ __device__ __forceinline__ void sell_slice(const LapView &L, const SpmmDev &a, c
     }
   }
   if constexpr (KIND != 3) {
-    const bool valid = row < L.n;
-    const int sd = valid ? sdeg[row] : 0xFF;
+    const bool valid = slot < L.n;
+    const int sd = valid ? sdeg[slot] : 0xFF;
     const int d = sd == 0xFF ? 0 : sd;
     const float *wp = W ? sw + __ldg(sptr + slice) + lane : nullptr;
     {
@@ -881,7 +884,7 @@ template <int LAP, typename TI, typename TT, int BP, bool W, int MODE, int KIND>
 __global__ void __launch_bounds__(128, SellOccupancy<TI, BP>::blocks)
 k_spmm_sell(const LapView L, const SpmmDev a, const int16_t *__restrict__ scol, const float *__restrict__ sw,
             const int64_t *__restrict__ sptr, const int64_t *__restrict__ cptr, const uint8_t *__restrict__ sdeg,
-            const int16_t *__restrict__ pcol, int ls) {
+            const int16_t *__restrict__ pcol, const uint16_t *__restrict__ srow, int ls) {
   if (a.done && *a.done) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (a.act_blocks) {
@@ -889,13 +892,13 @@ k_spmm_sell(const LapView L, const SpmmDev a, const int16_t *__restrict__ scol, 
     const int64_t items = 8 * static_cast<int64_t>(*a.n_act);
     for (int64_t i = blockIdx.x; i < items; i += gridDim.x) {
       const int64_t slice = static_cast<int64_t>(a.act_blocks[i >> 3]) * 32 + (i & 7) * 4 + wid;
-      sell_slice<LAP, TI, TT, BP, W, MODE, KIND>(L, a, scol, sw, sptr, cptr, sdeg, pcol, slice, lane);
+      sell_slice<LAP, TI, TT, BP, W, MODE, KIND>(L, a, scol, sw, sptr, cptr, sdeg, pcol, srow, slice, lane);
     }
     return;
   }
   const int64_t blk = blockIdx.x;
   const int64_t slice = ((blk >> ls) << (ls + 2)) + (blk & ((1 << ls) - 1)) + (static_cast<int64_t>(wid) << ls);
-  sell_slice<LAP, TI, TT, BP, W, MODE, KIND>(L, a, scol, sw, sptr, cptr, sdeg, pcol, slice, lane);
+  sell_slice<LAP, TI, TT, BP, W, MODE, KIND>(L, a, scol, sw, sptr, cptr, sdeg, pcol, srow, slice, lane);
 }
 
 // Staged blocks (SELL-32 with shared-pattern slices, unweighted graphs, L_C).
@@ -1338,29 +1341,32 @@ void spmm_launch_t(sphynx_graph *g, const SpmmDev &a) {
       const int ls = p.sell_ls;
       const unsigned gs = a.act_blocks ? static_cast<unsigned>(kListGrid)
                                        : static_cast<unsigned>(((warps + (int64_t{4} << ls) - 1) >> (ls + 2)) << ls);
-      const int16_t *sc = p.sell_col.as<int16_t>();
-      const float *swp = a.coef_sell ? a.coef_sell : p.sell_w.as<float>();
-      const int64_t *sp = p.sell_ptr.as<int64_t>();
-      const uint8_t *sd = p.sell_deg.as<uint8_t>();
+      const bool by_deg = std::is_same<TI, double>::value && p.variant == kSell32 && p.deg_row.p;
+      const int16_t *sc = (by_deg ? p.deg_col : p.sell_col).as<int16_t>();
+      const float *swp = a.coef_sell ? a.coef_sell : (by_deg ? p.deg_w : p.sell_w).as<float>();
+      const int64_t *sp = (by_deg ? p.deg_ptr : p.sell_ptr).as<int64_t>();
+      const int64_t *cp = (by_deg ? p.deg_cptr : p.sell_cptr).as<int64_t>();
+      const uint8_t *sd = (by_deg ? p.deg_deg : p.sell_deg).as<uint8_t>();
+      const uint16_t *srow = by_deg ? p.deg_row.as<uint16_t>() : nullptr;
       bool launched = p.variant == kSellPattern && spmm_launch_block<LAP, TI, TT, BP, W, MODE>(g, L, a);
       if constexpr (!W) {
         if (p.variant == kSellPattern && !launched) {
           const int64_t *pc = p.pat_cptr.as<int64_t>();
           const int16_t *pcl = p.pat_col.as<int16_t>();
           if (p.pat_all)
-            k_spmm_sell<LAP, TI, TT, BP, W, MODE, 3><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, pc, sd, pcl, ls);
+            k_spmm_sell<LAP, TI, TT, BP, W, MODE, 3><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, pc, sd, pcl, nullptr, ls);
           else
-            k_spmm_sell<LAP, TI, TT, BP, W, MODE, 2><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, pc, sd, pcl, ls);
+            k_spmm_sell<LAP, TI, TT, BP, W, MODE, 2><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, pc, sd, pcl, nullptr, ls);
           launched = true;
         }
       }
       if (!launched) {
-        if (p.sell_narrow == (g->n + 31) / 32)
-          k_spmm_sell<LAP, TI, TT, BP, W, MODE, 1><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, p.sell_cptr.as<int64_t>(),
-                                                                       sd, nullptr, ls);
+        if ((by_deg ? p.deg_narrow : p.sell_narrow) == (g->n + 31) / 32)
+          k_spmm_sell<LAP, TI, TT, BP, W, MODE, 1><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, cp,
+                                                                       sd, nullptr, srow, ls);
         else
-          k_spmm_sell<LAP, TI, TT, BP, W, MODE, 0><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, p.sell_cptr.as<int64_t>(),
-                                                                       sd, nullptr, ls);
+          k_spmm_sell<LAP, TI, TT, BP, W, MODE, 0><<<gs, 128, 0, st>>>(L, a, sc, swp, sp, cp,
+                                                                       sd, nullptr, srow, ls);
       }
     } else {
       const unsigned gsh = a.act_blocks ? static_cast<unsigned>(kListGrid) : static_cast<unsigned>(grid);
