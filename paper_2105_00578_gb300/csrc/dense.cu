@@ -388,13 +388,28 @@ k_lanczos_dots(const T *basis, int64_t ldv, int j1, const T *w, int64_t n, doubl
     for (int c = 0; c < kLzCols; ++c)
       if (c0 + c < j1) acc[c] = fma(basis[static_cast<int64_t>(c0 + c) * ldv + r], wv, acc[c]);
   }
+  // The warp's sums in double: a butterfly that halves the columns a lane holds
+  // at each of the first three steps (lane bits 4, 3, 2 choose the column), then
+  // two steps over the lanes of a column.  Nine FP64 additions a lane instead of
+  // 40: the FP64 pipe takes 64 cycles for each, and held half of the kernel's
+  // time (72 % busy; 40.7 -> 20.0 us a launch on average at n = 878,080).
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double d[kLzCols];
 #pragma unroll
-  for (int c = 0; c < kLzCols; ++c) {
-    double d = static_cast<double>(acc[c]);
-    for (int off = 16; off > 0; off >>= 1) d += __shfl_down_sync(0xffffffffu, d, off);
-    if (lane == 0) red[c][warp] = d;
+  for (int c = 0; c < kLzCols; ++c) d[c] = static_cast<double>(acc[c]);
+#pragma unroll
+  for (int half = kLzCols / 2, bit = 16; half >= 1; half >>= 1, bit >>= 1) {
+    const bool upper = lane & bit;
+#pragma unroll
+    for (int c = 0; c < kLzCols / 2; ++c) {
+      if (c >= half) break;
+      const double keep = upper ? d[c + half] : d[c], give = upper ? d[c] : d[c + half];
+      d[c] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+    }
   }
+  d[0] += __shfl_xor_sync(0xffffffffu, d[0], 2);
+  d[0] += __shfl_xor_sync(0xffffffffu, d[0], 1);
+  if ((lane & 3) == 0) red[lane >> 2][warp] = d[0];   // lane bits 4, 3, 2 spell the column
   __syncthreads();
   if (threadIdx.x < kLzCols && c0 + static_cast<int>(threadIdx.x) < j1) {
     double s = 0.0;
