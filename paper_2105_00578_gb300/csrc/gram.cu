@@ -16,8 +16,8 @@
 // lanes must all work: groups follow one another without regard to warps
 // (42 tiles at M = 24: 252 of 256 threads, where whole-warp groups left a third
 // idle), a slab is a whole number of rows for every group, and B S is formed once
-// per element, not once per tile.  n = 1,000,003, M = 24, B given: GRAM_OLD ->
-// GRAM_NEW us; the 672 FMAs a row alone take 1068 us.
+// per element, not once per tile.  n = 1,000,003, M = 24, B given: 2152 ->
+// 1180 us; the 672 FMAs a row alone take 1068 us.
 #include "internal.cuh"
 
 namespace sphynx {

@@ -253,7 +253,7 @@ __device__ __forceinline__ void cut_add(unsigned long long acc, unsigned long lo
 // Short rows and all part weights: a warp a 32-row slice, lane = row, over the
 // SELL-32 copy of the columns, whose entry t of the 32 rows is one segment (a
 // thread walking CSR entries of its own touches 32 lines a load: 350 us for the
-// 128^3 mesh, of which EVAL_US are left).  Lanes of one part add their weight once.
+// 128^3 mesh, of which 57 us are left).  Lanes of one part add their weight once.
 template <bool W>
 __global__ void __launch_bounds__(256)
 k_eval_short(const int16_t *__restrict__ scol, const float *__restrict__ sw, const int64_t *__restrict__ sptr,

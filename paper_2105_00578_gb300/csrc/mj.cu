@@ -24,10 +24,11 @@
 //    its 4096 points first so that it takes one global ticket a side; the last
 //    level writes the part ids instead.  The resulting sets (hence part ids) are
 //    exact and independent of scheduling.
-// 2,097,152 points, K = 64, six float dimensions: MJ_OLD -> MJ_NEW us.  Before, every
-// pass gathered its coordinates, 8-bit digits put nearly all points in a few
-// bins (a float's top eight bits are sign and exponent), and a warp took each
-// scatter ticket.
+// 2,097,152 points, K = 64, six float dimensions, with the evaluation of the cut
+// that follows: 2893 -> 976 us a call (707 us with the scratch kept in a pool).
+// Before, every pass gathered its coordinates, 8-bit digits put nearly all points
+// in a few bins (a float's top eight bits are sign and exponent), and a warp took
+// each scatter ticket.
 #include "internal.cuh"
 
 #include <cstring>
