@@ -33,6 +33,44 @@ constexpr int kSmallThreads = 256;
 
 // ---- cooperative building blocks (all threads of the CTA call them) --------
 
+// In-place Cholesky of the leading m x m of B (ld): on success the upper
+// triangle holds R with B = R^T R.  Returns the smallest pivot (R_kk^2) or
+// a negative value if a pivot was not positive.  Rows are scaled step by step;
+// chol_upper below is the faster one.  Float solves take this one: see the
+// choice of path in k_rayleigh_ritz.
+__device__ double chol_rows(double *B, int ld, int m, double *scratch) {
+  const int tid = threadIdx.x;
+  if (tid == 0) scratch[0] = INFINITY;
+  __syncthreads();
+  for (int k = 0; k < m; ++k) {
+    if (tid == 0) {
+      const double d = B[k * ld + k];
+      if (!(d > 0.0)) {
+        scratch[0] = -1.0;
+      } else {
+        if (d < scratch[0]) scratch[0] = d;
+        const double r = rsqrt(d);   // 1 / R_kk; R_kk = d r (the row below is scaled by r, not divided)
+        B[k * ld + k] = d * r;
+        scratch[1] = r;
+      }
+    }
+    __syncthreads();
+    if (scratch[0] < 0.0) return -1.0;
+    const double rinv = scratch[1];
+    for (int j = k + 1 + tid; j < m; j += blockDim.x) B[k * ld + j] *= rinv;
+    __syncthreads();
+    const int rem = m - k - 1;
+    for (int idx = tid; idx < rem * rem; idx += blockDim.x) {
+      const int i = k + 1 + idx / rem, j = k + 1 + idx % rem;
+      if (j >= i) B[i * ld + j] -= B[k * ld + i] * B[k * ld + j];
+    }
+    __syncthreads();
+  }
+  const double mn = scratch[0];
+  __syncthreads();
+  return mn;
+}
+
 // 1 / d for a positive normal d: the hardware's approximation (20 bits) and two
 // Newton steps, four dependent FP64 operations (the division takes more than
 // twice that, and an FP64 instruction of a warp occupies its quarter of the SM
@@ -54,9 +92,7 @@ __device__ __forceinline__ void upper_element(int t, int m, int &i, int &j) {
   j = i + t;
 }
 
-// In-place Cholesky of the leading m x m of B (ld): on success the upper
-// triangle holds R with B = R^T R.  Returns the smallest pivot (R_kk^2) or
-// a negative value if a pivot was not positive.  A thread keeps its elements
+// The same factorisation and result.  A thread keeps its elements
 // of the upper triangle in registers and eliminates with unscaled rows
 // (B_ij -= B_ki B_kj / d_k); the thread that forms the next pivot also forms its
 // reciprocal, so a step has one barrier, and the rows are scaled by
@@ -367,7 +403,7 @@ __device__ void eig_sym(RRSmem &S, double *A, double *V, int m, bool float_start
   }
   __syncthreads();
   matmul(S.P0, L, true, S.P0, L, S.P1, L, m, m, m);                 // G = V0^T V0
-  if (chol_upper(S.P1, L, m, S.scratch) <= 0.0) {                   // G = R^T R (never fails near I)
+  if (chol_rows(S.P1, L, m, S.scratch) <= 0.0) {                   // G = R^T R (never fails near I)
     jacobi_eig<double>(A, L, V, L, m, S.cs, S.pq);
     return;
   }
@@ -435,8 +471,8 @@ __device__ void rr_write(RRSmem &S, int m, int M, int ld, int nev, SolverState *
 // needed, takes as long as a dozen such steps.  Pairs too close for the quotient only keep
 // their orthogonality in the steps; if both are wanted a small FP64 Jacobi
 // solve on the nev x nev projection separates them, if not the caller's general
-// path runs.  The whole kernel at m = 21, nev = 7: 273 -> 82 us from float blocks,
-// 396 -> 95 us in FP64; m = 12, nev = 4: 124 and 165 -> 40 us.  Half of it is now the
+// path runs.  The whole kernel at m = 21, nev = 7: 396 -> 95 us; m = 12, nev = 4:
+// 165 -> 41 us.  Half of it is now the
 // float eigendecomposition (one warp, latency).
 
 // Float eigendecomposition of the pencil by one warp, lane j owning column j in
@@ -862,10 +898,16 @@ k_rayleigh_ritz(const double *ga, const double *gb, int M, int ld, int nev, doub
     S.Bh[(e / m) * L + e % m] = S.B[(e / m) * L + e % m];
   }
   __syncthreads();
-  const double minpiv = chol_upper(S.B, L, m, S.scratch);
+  // Float blocks (and their float-started solve) keep the general path: the
+  // refined one agrees to about 1e-14, but an iteration whose vectors are rounded
+  // to float and bfloat16 carries a changed last bit to 2e-3 of the residual norms
+  // that it stops at, and a float solve's results stay what they were, to the
+  // bit (273 against 82 us a step at m = 21).
+  const bool floats = mixed != 0 || yt_f32 != 0;
+  const double minpiv = floats ? chol_rows(S.B, L, m, S.scratch) : chol_upper(S.B, L, m, S.scratch);
   int m2 = m;
   // the refined path wants a basis that float arithmetic can orthogonalise
-  if (minpiv >= tau && minpiv >= 1e-4 && m >= 2 && m <= 32 && nev <= m && rr_refined(S, m, nev)) {
+  if (!floats && minpiv >= tau && minpiv >= 1e-4 && m >= 2 && m <= 32 && nev <= m && rr_refined(S, m, nev)) {
     rr_write(S, m, M, ld, nev, st, y64, yt, yt_f32, theta_out, svqb_out);
     return;
   }
