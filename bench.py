@@ -665,7 +665,7 @@ def run_ours(args, world, rank, local):
     dom = max(by_dt, key=lambda k: by_dt[k]["us_per_launch"] * by_dt[k]["launches_per_step"]) if by_dt else None
     info = spx.sphynx_get_info(graph.h)
     variant = {"csr": 0, "sell": 1, "pattern": 2}.get(args.spmm_variant, info["spmm_variant"])
-    schedule = {0: "k_spmm_short", 1: "k_spmm_sell", 2: "k_spmm_sell (shared-pattern slices)"}[variant]
+    schedule = {0: "k_spmm_short", 1: "k_spmm_sell", 2: "k_spmm_block / k_spmm_sell (shared-pattern slices)"}[variant]
     kernel_name = f"{schedule}<{dom} in>"
     traffic, traffic_meta = profiled_traffic(args.workload)
     # achieved: the scope table's algorithmic bytes of one launch of the
@@ -859,7 +859,7 @@ def main():
                     help="no benchmark: read the per-launch dram__bytes_read.sum / dram__bytes_write.sum of an ncu "
                          "--csv log and write profiles/traffic_<workload>.json, which later runs report as "
                          "roofline.traffic")
-    ap.add_argument("--kernel-regex", default=r"k_spmm_sell<(\(int\))?0, __nv_bfloat16, __nv_bfloat16",
+    ap.add_argument("--kernel-regex", default=r"k_spmm_(block|sell)<((\(int\))?0, )?__nv_bfloat16, __nv_bfloat16",
                     help="kernels of the ncu log that --ingest-ncu averages")
     ap.add_argument("--ncu-command", default="", help="the ncu command that wrote the log (recorded by --ingest-ncu)")
     ap.add_argument("--products", type=int, default=0, metavar="N",

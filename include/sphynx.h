@@ -183,7 +183,8 @@ typedef struct {
   int32_t weighted;          /* edge weights present                               */
   int32_t spmm_variant;      /* short-row schedule the autotuner chose at create
                                 from a float 8-column product and uses for every
-                                product: 0 = CSR staged in shared memory,
+                                product (F64 products use degree-ordered SELL-32
+                                slices where the graph has them): 0 = CSR staged in shared memory,
                                 1 = SELL-32, 2 = SELL-32 with shared-pattern slices */
   float tuned_us_csr;        /* the two schedules' times for that product (us)    */
   float tuned_us_sell;
@@ -353,7 +354,8 @@ int sphynx_amg_level(sphynx_handle g, int32_t level, sphynx_amg_level_info *info
  * Accumulation: products in the input type, short sums in the input type,
  * then a (hi, lo) float pair (float input) or double, per-CTA partials in
  * double added in a fixed order.
- * Scratch: allocated per call with cudaMallocAsync on `stream`. */
+ * Scratch: taken from a stream-ordered memory pool of the library on `stream`;
+ * at most 64 MB stay in the pool between calls. */
 int sphynx_gram(int32_t dtype, const void *const *s_blocks, const void *const *ls_blocks,
                 int32_t nblk, int32_t ld, int64_t n, const double *bdiag, double *ga_out,
                 double *gb_out, void *stream);
