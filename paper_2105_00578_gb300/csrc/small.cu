@@ -361,6 +361,7 @@ struct RRSmem {
   float V32[kMaxM * (kMaxM + 1)];
   float cs32[2 * kMaxM];
   float sel32[kMaxM];        // float reciprocal pivots of the refined path
+  float size32[2];           // its bounds on |W + s I| and |X|_F^2, see warp_pencil32
   int top;
   int pq32[2 * kMaxM];
   double d[kMaxM];
@@ -471,7 +472,18 @@ __device__ void rr_write(RRSmem &S, int m, int M, int ld, int nev, SolverState *
 // needed, takes as long as a dozen such steps.  Pairs too close for the quotient only keep
 // their orthogonality in the steps; if both are wanted a small FP64 Jacobi
 // solve on the nev x nev projection separates them, if not the caller's general
-// path runs.  The whole kernel at m = 21, nev = 7: 396 -> 95 us; m = 12, nev = 4:
+// path runs.
+// Which columns are wanted follows from the float values.  Where the nev-th and
+// the next are closer than those can be off, it is proved in the end: with X_u
+// the float basis of the unwanted columns and sigma the largest wanted value less
+// a few roundings, X_u^T (A - sigma B) X_u is positive definite only if no other
+// value lies below sigma (the wanted vectors' share of X_u adds a term that is not
+// negative).  It is nearly diagonal, so that its rows' sums nearly always decide;
+// otherwise its Cholesky factor does.  If there is none the general path runs.
+// (Vectors that do not couple, in diagonal pencils or decoupled blocks, leave no
+// other trace of a wrong order: every step is satisfied with them.)  The proof
+// takes 8 us at m = 21.
+// The whole kernel at m = 21, nev = 7: 396 -> 95 us; m = 12, nev = 4:
 // 165 -> 41 us.  Half of it is now the
 // float eigendecomposition (one warp, latency).
 
@@ -481,11 +493,12 @@ __device__ void rr_write(RRSmem &S, int m, int M, int ld, int nev, SolverState *
 // Jacobi rotations of L's columns (Hestenes; round-robin pairs, partner columns
 // read by shuffles) end in L J = U Sigma: U's columns are W's eigenvectors.  No
 // barriers and no shared traffic inside a sweep.  Returns X = R^{-1} U in
-// columns of x32 (ld), eigenvalues in lam.  Sweeps stop once every pair was
+// columns of x32 (ld), eigenvalues in lam, and in size32 a bound on |W + s I| and
+// |X|_F^2.  Sweeps stop once every pair was
 // within 1e-3 of orthogonal before its rotation (then 1e-6 after it).
 template <int MP>
 __device__ void warp_pencil32(const double *A, int ld, int m, double ascale, const float *x32, int ldx,
-                              float *lam, int *pq) {
+                              float *lam, int *pq, float *size32) {
   const int lane = threadIdx.x & 31;
   const bool in = lane < m;
   float own[MP];
@@ -623,10 +636,20 @@ __device__ void warp_pencil32(const double *A, int ld, int m, double ascale, con
     }
   }
   __syncwarp();
+  float xx = 0.f;
 #pragma unroll
-  for (int i = 0; i < MP; ++i)
-    if (i < m && in) t[i * ldx + lane] = own[i];
+  for (int i = 0; i < MP; ++i) {
+    if (i < m && in) {
+      t[i * ldx + lane] = own[i];
+      xx = fmaf(own[i], own[i], xx);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) xx += __shfl_xor_sync(0xffffffffu, xx, o);
   if (in) lam[lane] = nn - shift;
+  if (lane == 0) {
+    size32[0] = hi + shift;
+    size32[1] = xx;
+  }
 }
 
 // P0 = Q0 X_w and P1 = Q1 X_w (TRANS: Q^T X_w with one matrix and two blocks,
@@ -677,24 +700,32 @@ __device__ bool rr_refined(RRSmem &S, int m, int nev) {
   const double ascale = __hiloint2double((2046 - ex) << 20, 0);   // 2^(1023 - ex)
   if (tid < 32) {
     float *lam = S.V32;          // 32 values, then the m x m output
-    if (m <= 12) warp_pencil32<12>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32);
-    else if (m <= 24) warp_pencil32<24>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32);
-    else warp_pencil32<32>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32);
+    if (m <= 12) warp_pencil32<12>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32, S.size32);
+    else if (m <= 24) warp_pencil32<24>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32, S.size32);
+    else warp_pencil32<32>(S.A, L, m, ascale, S.A32, L32, lam, S.pq32, S.size32);
   }
   __syncthreads();
   const float *lam = S.V32, *x32 = S.V32 + 32;
+  int odd = 0;
   for (int i = tid; i < m; i += blockDim.x) {   // ascending order, stable
     const float li = lam[i];
+    odd |= !(fabsf(li) <= FLT_MAX);
     int rank = 0;
     for (int j = 0; j < m; ++j) rank += (lam[j] < li || (lam[j] == li && j < i)) ? 1 : 0;
     S.order[rank] = i;
     S.cs[rank] = static_cast<double>(li) / ascale;   // theta of every column, in order
   }
-  __syncthreads();
+  if (__syncthreads_or(odd)) return false;
   for (int e = tid; e < m * m; e += blockDim.x) {
     const int i = e / m, j = e % m;
     S.V[i * L + j] = static_cast<double>(x32[i * L32 + S.order[j]]);
   }
+  // The float values' error: a few roundings of |W + s I|, magnified by the
+  // condition |R|^2 |R^{-1}|^2 of the two triangular solves (trace B = m bounds |R|^2,
+  // |X|_F^2 is |R^{-1}|_F^2).  The largest error over random pencils of 3 to 32
+  // columns and basis conditions 1 to 100 is a fifteenth of this margin.
+  const float margin = 16 * 0x1p-24f * S.size32[0] * S.size32[1];
+  const bool clear = nev == m || (S.cs[nev] - S.cs[nev - 1]) * ascale > margin;   // uniform; false for NaN
   __syncthreads();
   int close = 0;
   for (int step = 0;; ++step) {
@@ -715,7 +746,9 @@ __device__ bool rr_refined(RRSmem &S, int m, int nev) {
       if (i != j) {
         const float num = static_cast<float>((S.W[i * L + j] + S.cs[j] * rij) * ascale);
         const float gap = static_cast<float>((S.cs[j] - S.cs[i]) * ascale);
-        if (fabsf(num) <= 1e-3f * fabsf(gap)) {
+        if (i >= nev && !(gap < 0.f)) {                 // not below an unwanted one, whatever their coupling
+          bad = 1;
+        } else if (fabsf(num) <= 1e-3f * fabsf(gap)) {
           e = static_cast<double>(num / gap);
         } else if (fabsf(num) > 4e-16f * m) {           // unresolved, and not rounding
           if (i < nev) pair = 1;
@@ -800,6 +833,32 @@ __device__ bool rr_refined(RRSmem &S, int m, int nev) {
     }
     if (tid < nev) S.qa[tid] = S.cs[tid];
     __syncthreads();
+  }
+  if (!clear) {
+    const int mu = m - nev;
+    const double sigma = S.qa[nev - 1] * ascale - 4.0 * m * 0x1p-53 * S.size32[0];
+    for (int e = tid; e < m * m; e += blockDim.x) {
+      const int o = (e / m) * L + e % m;
+      S.P2[o] = fma(-sigma, S.Bh[o], S.A[o] * ascale);
+    }
+    __syncthreads();
+    matmul(S.P2, L, false, S.V + nev, L, S.P0, L, m, m, mu);
+    for (int t = tid; t < mu * (mu + 1) / 2; t += blockDim.x) {
+      int i, j;
+      upper_element(t, mu, i, j);
+      double acc = 0.0;
+      for (int k = 0; k < m; ++k) acc = fma(S.V[k * L + nev + i], S.P0[k * L + j], acc);
+      S.W[i * L + j] = acc;
+      S.A32[i * L32 + j] = S.A32[j * L32 + i] = static_cast<float>(acc);
+    }
+    __syncthreads();
+    int dominant = 1;
+    for (int i = tid; i < mu; i += blockDim.x) {
+      float off = 0.f;
+      for (int j = 0; j < mu; ++j) off += j == i ? 0.f : fabsf(S.A32[i * L32 + j]);
+      dominant = S.A32[i * L32 + i] > 1.001f * off;      // false for NaN; 0.001: the float sums' rounding
+    }
+    if (!__syncthreads_and(dominant) && !(chol_upper(S.W, L, mu, S.scratch) > 0.0)) return false;
   }
   // sign as in the general path: w = R x, largest |entry| positive, first on ties
   for (int idx = tid; idx < m * nev; idx += blockDim.x) {
