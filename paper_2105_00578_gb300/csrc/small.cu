@@ -464,7 +464,8 @@ __device__ void rr_write(RRSmem &S, int m, int M, int ld, int nev, SolverState *
 // eigenvalue decomposition", 2018) in B-inner products and for the nev wanted
 // columns only: with X the current basis, S = X^T A X, R = I - X^T B X and
 // theta_j = S_jj / (1 - R_jj),
-//   x_j += sum_i x_i E_ij,  E_ij = (S_ij + theta_j R_ij) / (theta_j - theta_i),
+//   x_j += sum_i x_i E_ij,  E_ij = (S_ij + theta_j R_ij) / (theta_j - theta_i)
+//                                = R_ij / 2 + (S_ij + (theta_i + theta_j) R_ij / 2) / (theta_j - theta_i),
 // E_jj = R_jj / 2: a step costs 5 m^2 nev FP64 multiply-adds and squares the
 // error (a float eigendecomposition's 1e-6 -> 1e-11 -> below rounding).  FP64 is
 // what this kernel is short of (2 lanes a clock on the one SM it runs on): a
@@ -741,15 +742,22 @@ __device__ bool rr_refined(RRSmem &S, int m, int nev) {
     int big = 0, bad = 0, pair = 0;
     for (int idx = tid; idx < m * nev; idx += blockDim.x) {
       const int i = idx / nev, j = idx - (idx / nev) * nev;
-      const double rij = (i == j ? 1.0 : 0.0) - S.P2[i * L + j];
-      double e = 0.5 * rij;
+      // of two wanted columns both threads read the same elements and weight R_ij
+      // alike, so that their quotients cancel exactly and the pair's orthogonality
+      // takes R_ij alone: a quotient's error is its rounding noise over the gap.
+      // An unwanted column is not refined: its R_ij stays, and only the quotient
+      // with theta_j vanishes with the error.
+      const int o = i < j || i >= nev ? i * L + j : j * L + i;
+      const double rij = (i == j ? 1.0 : 0.0) - S.P2[o];
+      double e = i < nev ? 0.5 * rij : 0.0;
       if (i != j) {
-        const float num = static_cast<float>((S.W[i * L + j] + S.cs[j] * rij) * ascale);
+        const double weight = i < nev ? 0.5 * (S.cs[i] + S.cs[j]) : S.cs[j];
+        const float num = static_cast<float>((S.W[o] + weight * rij) * ascale);
         const float gap = static_cast<float>((S.cs[j] - S.cs[i]) * ascale);
         if (i >= nev && !(gap < 0.f)) {                 // not below an unwanted one, whatever their coupling
           bad = 1;
         } else if (fabsf(num) <= 1e-3f * fabsf(gap)) {
-          e = static_cast<double>(num / gap);
+          e += static_cast<double>(num / gap);
         } else if (fabsf(num) > 4e-16f * m) {           // unresolved, and not rounding
           if (i < nev) pair = 1;
           else bad = 1;
