@@ -31,6 +31,9 @@
  *   sphynx_create (a cudaStream_t, NULL = legacy default stream).  Calls that
  *   return results in host memory synchronise that stream before returning.
  *   A handle is not thread-safe; distinct handles may be used concurrently.
+ * - Waits inside kernels are bounded (about a second).  A product whose copies
+ *   to shared memory do not arrive by then leaves its output incomplete, and
+ *   the handle's next call that multiplies or returns results reports CUDA.
  */
 #ifndef SPHYNX_H
 #define SPHYNX_H

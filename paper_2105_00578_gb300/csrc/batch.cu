@@ -783,6 +783,7 @@ void batch_poly_setup_t(sphynx_graph *g, int k, int lap, uint64_t seed) {
   SPX_CUDA(cudaMemcpyAsync(hinv.data(), h, hinv.size() * 8, cudaMemcpyDeviceToHost, st));
   SPX_CUDA(cudaMemcpyAsync(herr.data(), err, herr.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
   SPX_CUDA(cudaStreamSynchronize(st));
+  check_fault(g);
   int kmax = k;
   for (int q = 0; q < count; ++q) {
     if (herr[q]) fail(SPHYNX_ERR_BREAKDOWN, "polynomial setup of graph %d: Lanczos tridiagonal not positive definite "
@@ -1228,6 +1229,7 @@ void batch_partition(sphynx_graph *g, int K, const sphynx_options *o, int32_t *d
     residual(X[1], LX[1], R);
     converge(0);
     SPX_CUDA(cudaStreamSynchronize(st));
+    check_fault(g);
 
     // the iteration body, captured once and repeated by a conditional WHILE node
     // (two bodies, one per ping-pong parity, so that a body is a fixed sequence)

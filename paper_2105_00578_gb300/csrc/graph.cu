@@ -1012,6 +1012,7 @@ void eval_partition(sphynx_graph *g, const int32_t *part, int K, double *cut, do
   std::vector<char> host(need);
   SPX_CUDA(cudaMemcpyAsync(host.data(), ws, need, cudaMemcpyDeviceToHost, g->stream));
   SPX_CUDA(cudaStreamSynchronize(g->stream));
+  check_fault(g);
   unsigned bad;
   memcpy(&bad, host.data() + 8, sizeof(bad));
   if (bad) fail(SPHYNX_ERR_INVALID_ARG, "part ids outside [0, K)");
@@ -1116,6 +1117,7 @@ int sphynx_create(const int64_t *row_ptr, const int32_t *col, const float *edge_
     g->jinv.alloc(n * sizeof(double));
     g->jinvf.alloc(n * sizeof(float));
     SPX_CUDA(cudaMallocHost(&g->host_flag, 256));
+    memset(g->host_flag, 0, 256);
 
     DevBuf gsb;
     gsb.alloc(sizeof(GraphStatsDev));

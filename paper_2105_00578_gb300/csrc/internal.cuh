@@ -308,7 +308,9 @@ struct sphynx_graph {
   std::map<std::string, sphynx::DevBuf> ws;  // named workspaces, grown on demand
   sphynx::Counters ctr;
   sphynx::DevBuf pinned_dummy;
-  void *host_flag = nullptr;                 // pinned int32[8] for convergence polls
+  void *host_flag = nullptr;                 // pinned int32[64]: [0] convergence polls, [32] the fault word
+  // set by a kernel whose bounded wait gave up (bounded_wait.cuh); check_fault reports it
+  int *fault() const { return static_cast<int *>(host_flag) + 32; }
   sphynx::BatchInfo batch;                   // set by sphynx_create_batch
   sphynx::AmgHierarchy *amg = nullptr;       // multigrid preconditioner (Sec. 5.3), built on demand
   sphynx::LapView view() const {
@@ -348,6 +350,9 @@ struct SpmmArgs {
   const int *n_act = nullptr;          // iterating (device list and count); NULL: every row
 };
 void spmm(sphynx_graph *g, const SpmmArgs &a);
+// Throws CUDA if a wait of an earlier launch gave up.  Every product calls it
+// first, and every call that returns results of products after its synchronisation.
+void check_fault(sphynx_graph *g);
 // both short-row schedules timed on this product (scratch outputs)
 SpmmTuning spmm_tune(sphynx_graph *g, const SpmmArgs &a);
 // every SELL slice stride timed on this product; sets plan.sell_ls to the fastest

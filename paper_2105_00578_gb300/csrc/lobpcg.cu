@@ -128,6 +128,7 @@ void poly_setup(sphynx_graph *g, const sphynx_options *o) {
   SPX_CUDA(cudaMemcpyAsync(g->poly_roots.data(), roots.p, kcap * sizeof(double), cudaMemcpyDeviceToHost, st));
   SPX_CUDA(cudaMemcpyAsync(herr, err.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   SPX_CUDA(cudaStreamSynchronize(st));
+  check_fault(g);
   if (herr[0]) fail(SPHYNX_ERR_BREAKDOWN, "polynomial setup: Lanczos tridiagonal not positive definite (%d)", herr[0]);
   g->poly_roots.resize(herr[1]);
   g->poly_k = herr[1];
@@ -355,6 +356,7 @@ EigenResult lobpcg(sphynx_graph *g, const sphynx_options *o, int b, const double
   SolverState hs;
   SPX_CUDA(cudaMemcpyAsync(&hs, state, sizeof(hs), cudaMemcpyDeviceToHost, st));
   SPX_CUDA(cudaStreamSynchronize(st));
+  check_fault(g);
   EigenResult r;
   r.iterations = hs.iters;
   r.svqb = hs.svqb_steps;
@@ -589,6 +591,7 @@ int sphynx_precond_setup(sphynx_handle g, const sphynx_options *opt, double *roo
     check_options(g, opt);
     if (opt->precond == SPHYNX_PRECOND_AMG) {
       amg_setup(g, opt->seed, true);
+      check_fault(g);
       return SPHYNX_OK;
     }
     if (opt->precond != SPHYNX_PRECOND_POLY) return SPHYNX_OK;

@@ -95,7 +95,8 @@ SpmmDev tune_args(sphynx_graph *g, const SpmmArgs &a) {
     s.t_out = base + out_bytes;
   }
   return SpmmDev{s.x,      s.ld_x, s.ld_y, s.y,     s.t_out,      s.yacc,       s.first,   s.yterms,
-                 s.inv,    s.invf, s.i_cur, nullptr, s.row_graph, s.inv_stride, nullptr, nullptr, s.x, nullptr, nullptr};
+                 s.inv,    s.invf, s.i_cur, nullptr, s.row_graph, s.inv_stride, nullptr, nullptr, s.x, nullptr, nullptr,
+                 g->fault()};
 }
 
 }  // namespace
@@ -130,6 +131,7 @@ SpmmTuning spmm_tune(sphynx_graph *g, const SpmmArgs &a) {
       t.us[v] = ms * 1000.f < t.us[v] ? ms * 1000.f : t.us[v];
     }
   }
+  check_fault(g);               // the last event was waited for
   g->ctr.launches = launches;   // tuning launches are not part of the caller's work
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -171,6 +173,7 @@ void spmm_tune_sell_stride(sphynx_graph *g, const SpmmArgs &a) {
       us[ls] = ms * 1000.f < us[ls] ? ms * 1000.f : us[ls];
     }
   }
+  check_fault(g);
   g->ctr.launches = launches;
   g->plan.variant = variant;
   cudaEventDestroy(e0);
@@ -183,7 +186,15 @@ void spmm_tune_sell_stride(sphynx_graph *g, const SpmmArgs &a) {
   g->plan.sell_ls = best;
 }
 
+void check_fault(sphynx_graph *g) {
+  volatile int *f = g->fault();
+  if (!*f) return;
+  *f = 0;
+  fail(SPHYNX_ERR_CUDA, "a product's copies to shared memory did not arrive in time; its output is incomplete");
+}
+
 void spmm(sphynx_graph *g, const SpmmArgs &a) {
+  check_fault(g);
   if (!(a.bp == 1 || a.bp == 4 || a.bp == 8 || a.bp == 12 || a.bp == 16))
     fail(SPHYNX_ERR_INVALID_ARG, "spmm: block width %d", a.bp);
   // the kernels index X (and the chain's output) with the compile-time width:
@@ -204,7 +215,8 @@ void spmm(sphynx_graph *g, const SpmmArgs &a) {
   if (a.mode == 1 && (a.yterms < 0 || a.yterms > 2 || (a.first && a.yterms != 2)))
     fail(SPHYNX_ERR_INVALID_ARG, "spmm: polynomial step adds 0, 1 or 2 terms (2 on the first step)");
   SpmmDev d{a.x,   a.ld_x, a.ld_y, a.y,      a.t_out,    a.yacc,        a.first,  a.yterms,
-            a.inv, a.invf, a.i_cur, a.done, a.row_graph, a.inv_stride, a.act_blocks, a.n_act, a.x, nullptr, nullptr};
+            a.inv, a.invf, a.i_cur, a.done, a.row_graph, a.inv_stride, a.act_blocks, a.n_act, a.x, nullptr, nullptr,
+            g->fault()};
   const bool prescaled = g->plan.prescale && a.lap == SPHYNX_NORMALIZED && a.tin != DT::BF16 && g->n > 0;
   const bool coefs = g->plan.prescale && a.lap == SPHYNX_NORMALIZED && a.tin == DT::BF16 && g->n > 0;
   if (coefs) {

@@ -26,6 +26,7 @@
 // whichever step adds them.
 #pragma once
 
+#include "bounded_wait.cuh"
 #include "internal.cuh"
 
 namespace sphynx {
@@ -166,6 +167,7 @@ struct SpmmDev {              // kernel-side view of SpmmArgs
   const void *xe;            // the epilogue's own rows X_i (x itself, or X when x holds D^{-1/2} X)
   const float *coef_csr;     // normalized: per-entry (w_ij or 1) D^{-1/2}_j in CSR order (NULL: gather D^{-1/2}_j)
   const float *coef_sell;    // the same in SELL slot order
+  int *fault;                // the handle's fault word (host memory): set where a bounded wait gave up
 };
 
 constexpr int kListGrid = kSmCount * 16;   // CTAs of a launch that walks an active-block list
@@ -1056,22 +1058,6 @@ __device__ __forceinline__ void staged_run(const unsigned char *p, int rot, cons
   }
 }
 
-// waits for the first phase of an mbarrier; false after 2^16 tries (each of
-// them a hardware wait of its own), which the copies of a block never need:
-// the caller then reads global memory instead
-__device__ __forceinline__ bool staged_wait(unsigned bar32) {
-  for (int tries = 0; tries < (1 << 16); ++tries) {
-    unsigned ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok)
-                 : "r"(bar32)
-                 : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
 // Descriptor of a block (kBlkDesc ints): [0] ranges, [1] runs, [2] staged row of
 // the block's row 0; then per range {first row relative to the block's, rows,
 // staged row}; then per run: staged row | length << 16 | first mask bit << 18.
@@ -1122,7 +1108,7 @@ k_spmm_block(const LapView L, const SpmmDev a, const int32_t *__restrict__ desc,
   }
   __syncthreads();   // expectations and plain stores first
   if (tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar32) : "memory");
-  const bool landed = staged_wait(bar32);
+  if (!bounded_wait_or_fault(bar32, a.fault)) return;   // whole warps; no block barrier follows
   const int rot = B::nq == 2 ? (tid >> 2) & 1 : (B::nq == 4 ? (tid >> 1) & 3 : 0);
   const unsigned char *mine = staged + tid * (kBlkRows * rb);
   const int *runs = sd + 3 + 3 * nrange;
@@ -1144,7 +1130,7 @@ k_spmm_block(const LapView L, const SpmmDev a, const int32_t *__restrict__ desc,
 #pragma unroll
     for (int c = 0; c < BP; ++c) chk += sum[j][c];
   }
-  if (__any_sync(kFull, chk != chk || !landed)) {
+  if (__any_sync(kFull, chk != chk)) {
 #pragma unroll
     for (int j = 0; j < kBlkRows; ++j)
 #pragma unroll
@@ -1167,7 +1153,6 @@ k_spmm_block(const LapView L, const SpmmDev a, const int32_t *__restrict__ desc,
           for (int c = 0; c < BP; ++c) sum[j][c] += v[c];
         }
     }
-    if (!landed) (void)staged_wait(bar32);   // copies still in flight write to this block's memory
   }
 #pragma unroll
   for (int j = 0; j < kBlkRows; ++j) {
@@ -1186,8 +1171,7 @@ k_spmm_block(const LapView L, const SpmmDev a, const int32_t *__restrict__ desc,
       }
     }
     StagedRow<TI, BP> r;
-    if (landed) r.load(mine + (sd[2] + j) * rb, 0);
-    else r.load(x + (r0 + kBlkRows * tid + j) * rb, 0);
+    r.load(mine + (sd[2] + j) * rb, 0);
     staged_values<TI, BP>(r, xi);
     spmm_epilogue<SPHYNX_COMBINATORIAL, TI, TT, BP, MODE>(L, a, r0 + kBlkRows * tid + j, xi, ord);
   }
