@@ -71,17 +71,6 @@ __device__ double chol_rows(double *B, int ld, int m, double *scratch) {
   return mn;
 }
 
-// 1 / d for a positive normal d: the hardware's approximation (20 bits) and two
-// Newton steps, four dependent FP64 operations (the division takes more than
-// twice that, and an FP64 instruction of a warp occupies its quarter of the SM
-// for 64 cycles)
-__device__ __forceinline__ double recip_newton(double d) {
-  double x;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
-  x = fma(x, fma(-d, x, 1.0), x);
-  return fma(x, fma(-d, x, 1.0), x);
-}
-
 // element t of the row-major upper triangle of an m x m matrix
 __device__ __forceinline__ void upper_element(int t, int m, int &i, int &j) {
   i = 0;
@@ -117,7 +106,7 @@ __device__ double chol_upper(double *B, int ld, int m, double *scratch) {
   }
   if (tid == 0) {
     piv[0] = v[0];
-    rec[0] = recip_newton(v[0]);
+    rec[0] = __drcp_rn(v[0]);
   }
   __syncthreads();
   double mn = INFINITY;
@@ -135,7 +124,7 @@ __device__ double chol_upper(double *B, int ld, int m, double *scratch) {
         B[ei[u] * ld + ej[u]] = v[u];
         if (ej[u] == k + 1) {        // the next pivot
           piv[k + 1] = v[u];
-          rec[k + 1] = recip_newton(v[u]);
+          rec[k + 1] = __drcp_rn(v[u]);
         }
       }
     }
