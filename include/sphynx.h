@@ -186,9 +186,12 @@ typedef struct {
   int32_t weighted;          /* edge weights present                               */
   int32_t spmm_variant;      /* short-row schedule the autotuner chose at create
                                 from a float 8-column product and uses for every
-                                product (F64 products use degree-ordered SELL-32
-                                slices where the graph has them): 0 = CSR staged in shared memory,
-                                1 = SELL-32, 2 = SELL-32 with shared-pattern slices */
+                                product that can: 0 = CSR staged in shared memory,
+                                1 = SELL-32, 2 = SELL-32 with shared-pattern slices.
+                                Where 2 means staged blocks, F64 and normalized
+                                products take the fastest of the other kernels
+                                (sphynx_plan_info), and F64 products use degree-
+                                ordered SELL-32 slices where the graph has them   */
   float tuned_us_csr;        /* the two schedules' times for that product (us)    */
   float tuned_us_sell;
   int64_t sell_slices;       /* SELL-32 slices (32 rows each)                      */
@@ -215,6 +218,20 @@ typedef struct {
                                 that union once per slice plus a 32-bit entry mask
                                 per row instead of one offset per entry           */
 } sphynx_graph_info;
+
+/* How a handle's products run, for tests and profiling. */
+typedef struct {
+  int32_t staged_threads;    /* threads of a staged block (three rows each); 0: the
+                                graph has none                                      */
+  int32_t staged_rows;       /* rows of X the largest block stages                 */
+  int32_t staged_used;       /* the autotuner chose them for the products that can  */
+  int32_t lane_variant;      /* schedule of the products that cannot (spmm_variant
+                                where nothing is staged)                            */
+  int32_t degree_slices;     /* F64 products use degree-ordered slices              */
+  float tuned_us_staged;     /* staged float 8-column product (us); 0: not timed    */
+  float tuned_us_stride[5];  /* the lane-per-row SELL kernel at slice strides 1, 2,
+                                4, 8, 16; 0: not timed                              */
+} sphynx_plan_info;
 
 /* Fill *opt with the defaults listed in sphynx_options. */
 void sphynx_default_options(sphynx_options *opt);
@@ -248,6 +265,9 @@ void sphynx_destroy(sphynx_handle g);
 
 /* Sizes and degree statistics of the graph (host struct). */
 int sphynx_get_info(sphynx_handle g, sphynx_graph_info *info);
+
+/* How the handle's products run (host struct). */
+int sphynx_get_plan_info(sphynx_handle g, sphynx_plan_info *info);
 
 /* Pin the short-row SpMM schedule of the handle: 0 = CSR staged in shared
  * memory, 1 = SELL-32, 2 = SELL-32 with shared-pattern slices (only when the

@@ -77,6 +77,12 @@ class GraphInfo(C.Structure):
                 ("tuned_us_pattern", C.c_float), ("sell_pattern_slices", C.c_int64)]
 
 
+class PlanInfo(C.Structure):
+    _fields_ = [("staged_threads", C.c_int32), ("staged_rows", C.c_int32), ("staged_used", C.c_int32),
+                ("lane_variant", C.c_int32), ("degree_slices", C.c_int32), ("tuned_us_staged", C.c_float),
+                ("tuned_us_stride", C.c_float * 5)]
+
+
 class AmgLevelInfo(C.Structure):
     _fields_ = [("levels", C.c_int32), ("reserved", C.c_int32), ("n", C.c_int64), ("nnz", C.c_int64),
                 ("n_next", C.c_int64), ("lambda_max", C.c_double)]
@@ -94,6 +100,7 @@ def _load():
         "sphynx_create": (C.c_int, [vp, vp, vp, vp, i64, i64, u32, vp, C.POINTER(vp)]),
         "sphynx_destroy": (None, [vp]),
         "sphynx_get_info": (C.c_int, [vp, C.POINTER(GraphInfo)]),
+        "sphynx_get_plan_info": (C.c_int, [vp, C.POINTER(PlanInfo)]),
         "sphynx_set_spmm_variant": (C.c_int, [vp, i32]),
         "sphynx_set_spmm_sell_stride": (C.c_int, [vp, i32]),
         "sphynx_degrees": (C.c_int, [vp, vp]),
@@ -222,6 +229,14 @@ def sphynx_get_info(h) -> dict:
     info = GraphInfo()
     check(LIB.sphynx_get_info(h, C.byref(info)))
     return {f: getattr(info, f) for f, _ in info._fields_}
+
+
+def sphynx_get_plan_info(h) -> dict:
+    info = PlanInfo()
+    check(LIB.sphynx_get_plan_info(h, C.byref(info)))
+    out = {f: getattr(info, f) for f, _ in info._fields_}
+    out["tuned_us_stride"] = list(info.tuned_us_stride)
+    return out
 
 
 def sphynx_set_spmm_variant(h, variant: int) -> None:

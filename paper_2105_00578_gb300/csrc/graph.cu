@@ -914,10 +914,11 @@ void build_blocks(sphynx_graph *g) {
   p.blk_staged_rows = h[1];
 }
 
-// The short-row schedule is a property of the graph's structure: both are
-// timed at create on a float 8-column product and the faster serves every
-// later product of the handle.
-// The autotuner: at create, times both short-row schedules and, on graphs with
+// The short-row schedule is a property of the graph's structure: all are
+// timed at create on a float 8-column product and the fastest serves every
+// later product of the handle that can use it, the fastest lane-per-row one the
+// others.
+// The autotuner: at create, times the short-row schedules and, on graphs with
 // rows longer than kShortDeg, the medium-row ceilings {kShortDeg, 128, kMedDeg}
 // on a float 8-column product, and keeps the fastest combination; when that is
 // SELL-32, it then times the slice strides 1 .. 16 and keeps the fastest.
@@ -954,7 +955,7 @@ void autotune_spmm(sphynx_graph *g, const int64_t *host_rowptr) {
   for (int c : ceilings) {
     if (ceilings.size() > 1) build_plan(g, rp, c);
     const SpmmTuning t = spmm_tune(g, a);
-    const float us = t.us[t.variant];
+    const float us = std::min(t.us[t.variant], t.us_staged);
     if (us < best) {
       best = us;
       best_ceiling = c;
@@ -962,9 +963,13 @@ void autotune_spmm(sphynx_graph *g, const int64_t *host_rowptr) {
     }
   }
   if (ceilings.size() > 1 && best_ceiling != ceilings.back()) build_plan(g, rp, best_ceiling);
-  g->plan.tuned_variant = best_t.variant;
+  g->plan.lane_variant = best_t.variant;
+  g->plan.tuned_staged = best_t.staged;
+  g->plan.tuned_us_staged = best_t.us_staged < 1e30f ? best_t.us_staged : 0.f;
+  g->plan.tuned_variant = best_t.staged ? static_cast<int>(kSellPattern) : best_t.variant;
   for (int v = 0; v < kSpmmVariants; ++v) g->plan.tuned_us[v] = best_t.us[v];
   for (float &u : g->plan.tuned_ls_us) u = 0.f;
+  // strides serve what does not stage: FP64 and normalized products among others
   if (best_t.variant != kCsrStaged) spmm_tune_sell_stride(g, a);
   SPX_CUDA(cudaStreamSynchronize(g->stream));
 }
@@ -1199,7 +1204,9 @@ int sphynx_get_info(sphynx_handle g, sphynx_graph_info *info) {
     info->spmm_variant = g->plan.tuned_variant;
     info->tuned_us_csr = g->plan.tuned_us[kCsrStaged];
     info->tuned_us_sell = g->plan.tuned_us[kSell32];
-    info->tuned_us_pattern = g->plan.pat_slices > 0 ? g->plan.tuned_us[kSellPattern] : 0.f;
+    info->tuned_us_pattern = g->plan.pat_slices == 0 ? 0.f
+                             : g->plan.tuned_staged && g->plan.tuned_us_staged > 0.f ? g->plan.tuned_us_staged
+                                                                                     : g->plan.tuned_us[kSellPattern];
     info->sell_pattern_slices = g->plan.pat_slices;
     info->regular = g->max_degree * g->n <= 10 * g->nnz ? 1 : 0;
     info->spmm_med_max = g->plan.med_max;
@@ -1213,6 +1220,22 @@ int sphynx_get_info(sphynx_handle g, sphynx_graph_info *info) {
                                         : 8.0 * static_cast<double>(g->n + 1) +
                                               g->plan.short_entries * (g->weighted ? 8.0 : 4.0)) +
                              g->plan.med_bytes + g->plan.long_bytes;
+    return SPHYNX_OK;
+  });
+}
+
+int sphynx_get_plan_info(sphynx_handle g, sphynx_plan_info *info) {
+  return guarded([&]() -> int {
+    if (!g || !info) fail(SPHYNX_ERR_INVALID_ARG, "NULL argument");
+    memset(info, 0, sizeof(*info));
+    const SpmmPlan &p = g->plan;
+    info->staged_threads = p.blk_threads;
+    info->staged_rows = p.blk_threads ? p.blk_staged_rows : 0;
+    info->staged_used = p.blk_threads && p.tuned_staged ? 1 : 0;
+    info->lane_variant = p.lane_variant;
+    info->degree_slices = p.deg_row.p ? 1 : 0;
+    info->tuned_us_staged = p.tuned_us_staged;
+    for (int k = 0; k < kSellLsCount; ++k) info->tuned_us_stride[k] = p.tuned_ls_us[k];
     return SPHYNX_OK;
   });
 }

@@ -129,15 +129,21 @@ __device__ __forceinline__ int64_t sell_slot_row(const uint16_t *order, int64_t 
 }
 
 struct SpmmTuning {
-  int variant;
+  int variant;                       // the fastest lane-per-row schedule
+  bool staged;                       // staged blocks are faster still
   float us[kSpmmVariants];           // measured time of each schedule (1e30: not available)
+  float us_staged;                   // and of the staged blocks
 };
 
 struct SpmmPlan {
   int variant = kCsrStaged;          // schedule of the launch being issued
   int forced = -1;                   // >= 0: every product uses this schedule
-  int tuned_variant = kCsrStaged;    // the autotuner's choice for this graph
-  float tuned_us[kSpmmVariants] = {0.f, 0.f, 0.f};   // its timings of the schedules
+  int tuned_variant = kCsrStaged;    // the autotuner's choice for this graph: kSellPattern where staged
+  bool tuned_staged = false;         // blocks won, which the products that cannot use them
+  int lane_variant = kCsrStaged;     // replace by the fastest lane-per-row schedule
+  bool stage_now = false;            // the launch being issued uses the staged blocks
+  float tuned_us[kSpmmVariants] = {0.f, 0.f, 0.f};   // its timings of the lane-per-row schedules
+  float tuned_us_staged = 0.f;       // and of the staged blocks
   int sell_ls = 0;                   // SELL blocks: warps take slices 2^sell_ls apart
   float tuned_ls_us[kSellLsCount] = {};   // the autotuner's time for each sell_ls
   DevBuf tune_scratch;
@@ -353,7 +359,7 @@ void spmm(sphynx_graph *g, const SpmmArgs &a);
 // Throws CUDA if a wait of an earlier launch gave up.  Every product calls it
 // first, and every call that returns results of products after its synchronisation.
 void check_fault(sphynx_graph *g);
-// both short-row schedules timed on this product (scratch outputs)
+// the short-row schedules timed on this product (scratch outputs)
 SpmmTuning spmm_tune(sphynx_graph *g, const SpmmArgs &a);
 // every SELL slice stride timed on this product; sets plan.sell_ls to the fastest
 void spmm_tune_sell_stride(sphynx_graph *g, const SpmmArgs &a);

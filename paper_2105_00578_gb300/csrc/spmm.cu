@@ -99,61 +99,88 @@ SpmmDev tune_args(sphynx_graph *g, const SpmmArgs &a) {
                  g->fault()};
 }
 
+// can this product use the graph's staged blocks (k_spmm_block)?
+bool blocks_take(const sphynx_graph *g, const SpmmArgs &a) {
+  return g->plan.blk_threads > 0 && !g->weighted && a.lap != SPHYNX_NORMALIZED && a.tin != DT::F64 && a.bp > 1 &&
+         !a.act_blocks && reinterpret_cast<uintptr_t>(a.x) % 16 == 0 &&
+         static_cast<size_t>(g->plan.blk_staged_rows) * a.bp * dt_size(a.tin) <= kBlkSmemMax;
+}
+
+struct TuneEvents {
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  TuneEvents() {
+    SPX_CUDA(cudaEventCreate(&e0));
+    SPX_CUDA(cudaEventCreate(&e1));
+  }
+  ~TuneEvents() {
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+  }
+  // microseconds of one launch
+  float time(sphynx_graph *g, const SpmmArgs &a, const SpmmDev &d) {
+    SPX_CUDA(cudaEventRecord(e0, g->stream));
+    dispatch(g, a, d);
+    SPX_CUDA(cudaEventRecord(e1, g->stream));
+    SPX_CUDA(cudaEventSynchronize(e1));
+    float ms = 0.f;
+    SPX_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+    return ms * 1000.f;
+  }
+};
+
 }  // namespace
 
-// Time both short-row schedules for this product with the caller's input
-// and scratch outputs, alternating them over five rounds, and return the
-// faster.
+// Time the short-row schedules for this product with the caller's input and
+// scratch outputs, alternating them over five rounds: the lane-per-row kernels
+// of every layout, and the staged blocks where the product can use them.
 SpmmTuning spmm_tune(sphynx_graph *g, const SpmmArgs &a) {
-  const SpmmArgs &s = a;
   const SpmmDev d = tune_args(g, a);
-  cudaEvent_t e0, e1;
-  SPX_CUDA(cudaEventCreate(&e0));
-  SPX_CUDA(cudaEventCreate(&e1));
-  SpmmTuning t{kCsrStaged, {1e30f, 1e30f, 1e30f}};
+  TuneEvents ev;
+  SpmmTuning t{kCsrStaged, false, {1e30f, 1e30f, 1e30f}, 1e30f};
   const int64_t launches = g->ctr.launches;
   const int nv = g->plan.pat_slices > 0 ? 3 : 2;   // the shared-pattern layout exists on some graphs only
-  for (int v = 0; v < nv; ++v) {   // warm-up of each
-    g->plan.variant = v;
-    dispatch(g, s, d);
+  const bool blocks = blocks_take(g, a);           // candidate nv
+  const int nc = nv + (blocks ? 1 : 0);
+  auto pick = [&](int v) {
+    g->plan.stage_now = v == nv;
+    g->plan.variant = v == nv ? static_cast<int>(kSellPattern) : v;
+  };
+  for (int v = 0; v < nc; ++v) {   // warm-up of each
+    pick(v);
+    dispatch(g, a, d);
   }
   // alternate the schedules so that neither always runs on a warmer L2
   for (int round = 0; round < 5; ++round) {
-    for (int k = 0; k < nv; ++k) {
-      const int v = (round + k) % nv;
-      g->plan.variant = v;
-      SPX_CUDA(cudaEventRecord(e0, g->stream));
-      dispatch(g, s, d);
-      SPX_CUDA(cudaEventRecord(e1, g->stream));
-      SPX_CUDA(cudaEventSynchronize(e1));
-      float ms = 0.f;
-      SPX_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      t.us[v] = ms * 1000.f < t.us[v] ? ms * 1000.f : t.us[v];
+    for (int k = 0; k < nc; ++k) {
+      const int v = (round + k) % nc;
+      pick(v);
+      float &us = v == nv ? t.us_staged : t.us[v];
+      us = std::min(us, ev.time(g, a, d));
     }
   }
   check_fault(g);               // the last event was waited for
   g->ctr.launches = launches;   // tuning launches are not part of the caller's work
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  t.variant = kCsrStaged;
+  g->plan.stage_now = false;
   for (int v = 1; v < nv; ++v)
     if (t.us[v] < t.us[t.variant]) t.variant = v;
+  // blocks too wide for this product may still serve narrower ones: with the layout's own result
+  t.staged = blocks ? t.us_staged < t.us[t.variant] : g->plan.blk_threads > 0 && t.variant == kSellPattern;
   return t;
 }
 
 // Time the SELL schedule under every slice stride 2^ls (ls < kSellLsCount),
 // rotating the order over five rounds, and keep the fastest in plan.sell_ls.
-// Strides change only which block runs a slice, never a product's value.
+// Strides change only which block runs a slice, never a product's value, and
+// mean nothing to staged blocks: the lane-per-row kernel is timed.
 void spmm_tune_sell_stride(sphynx_graph *g, const SpmmArgs &a) {
   const SpmmDev d = tune_args(g, a);
-  cudaEvent_t e0, e1;
-  SPX_CUDA(cudaEventCreate(&e0));
-  SPX_CUDA(cudaEventCreate(&e1));
+  TuneEvents ev;
   const int64_t launches = g->ctr.launches;
   const int variant = g->plan.variant;
   // the SELL schedule in force (pinned, else tuned); plain SELL-32 when that is CSR
-  const int sv = g->plan.forced > 0 ? g->plan.forced : g->plan.tuned_variant;
+  const int sv = g->plan.forced > 0 ? g->plan.forced : g->plan.lane_variant;
   g->plan.variant = sv == kSellPattern ? kSellPattern : kSell32;
+  g->plan.stage_now = false;
   float us[kSellLsCount];
   for (int k = 0; k < kSellLsCount; ++k) {   // warm-up of each
     us[k] = 1e30f;
@@ -164,20 +191,12 @@ void spmm_tune_sell_stride(sphynx_graph *g, const SpmmArgs &a) {
     for (int k = 0; k < kSellLsCount; ++k) {
       const int ls = (round + k) % kSellLsCount;
       g->plan.sell_ls = ls;
-      SPX_CUDA(cudaEventRecord(e0, g->stream));
-      dispatch(g, a, d);
-      SPX_CUDA(cudaEventRecord(e1, g->stream));
-      SPX_CUDA(cudaEventSynchronize(e1));
-      float ms = 0.f;
-      SPX_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      us[ls] = ms * 1000.f < us[ls] ? ms * 1000.f : us[ls];
+      us[ls] = std::min(us[ls], ev.time(g, a, d));
     }
   }
   check_fault(g);
   g->ctr.launches = launches;
   g->plan.variant = variant;
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
   int best = 0;
   for (int k = 0; k < kSellLsCount; ++k) {
     g->plan.tuned_ls_us[k] = us[k];
@@ -229,8 +248,11 @@ void spmm(sphynx_graph *g, const SpmmArgs &a) {
   // from a float product.  Double products take the degree-ordered slices
   // wherever those exist (300,000-vertex geometric graph, 4 columns, a chain
   // step: 59.5 us in the CSR schedule, 39.2 in these).
-  g->plan.variant = g->plan.forced >= 0 ? g->plan.forced
-                    : a.tin == DT::F64 && g->plan.deg_row.p ? static_cast<int>(kSell32) : g->plan.tuned_variant;
+  SpmmPlan &p = g->plan;
+  p.stage_now = (p.forced >= 0 ? p.forced == kSellPattern : p.tuned_staged) && blocks_take(g, a);
+  p.variant = p.forced >= 0 ? p.forced
+              : p.stage_now ? static_cast<int>(kSellPattern)
+              : a.tin == DT::F64 && p.deg_row.p ? static_cast<int>(kSell32) : p.lane_variant;
 
   // algorithmic bytes: the graph in the layout the schedule reads (CSR row
   // pointers and indices, or the SELL-32 slices plus the long rows' CSR

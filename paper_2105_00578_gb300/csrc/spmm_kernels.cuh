@@ -1177,15 +1177,16 @@ k_spmm_block(const LapView L, const SpmmDev a, const int32_t *__restrict__ desc,
   }
 }
 
-// launches the staged-block kernel when this product qualifies
+// launches the staged-block kernel when this product is to use it (spmm() and
+// the autotuner decide, blocks_take())
 template <int LAP, typename TI, typename TT, int BP, bool W, int MODE>
 bool spmm_launch_block(sphynx_graph *g, const LapView &L, const SpmmDev &a) {
   if constexpr (W || LAP == SPHYNX_NORMALIZED || std::is_same<TI, double>::value || BP == 1) {
     return false;
   } else {
     const SpmmPlan &p = g->plan;
+    if (!p.stage_now) return false;
     const size_t smem = static_cast<size_t>(p.blk_staged_rows) * BlockTraits<TI, BP>::row_bytes;
-    if (p.blk_threads == 0 || a.act_blocks || smem > kBlkSmemMax || reinterpret_cast<uintptr_t>(a.x) % 16) return false;
     SPX_CUDA(cudaFuncSetAttribute(k_spmm_block<TI, TT, BP, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(kBlkSmemMax)));
     const int64_t rows = static_cast<int64_t>(kBlkRows) * p.blk_threads;
