@@ -189,7 +189,8 @@ typedef struct {
                                 product that can: 0 = CSR staged in shared memory,
                                 1 = SELL-32, 2 = SELL-32 with shared-pattern slices.
                                 Where 2 means staged blocks, F64 and normalized
-                                products take the fastest of the other kernels
+                                products and the widths and steps that gain nothing
+                                from them take the fastest of the other kernels
                                 (sphynx_plan_info), and F64 products use degree-
                                 ordered SELL-32 slices where the graph has them   */
   float tuned_us_csr;        /* the two schedules' times for that product (us)    */
@@ -224,7 +225,9 @@ typedef struct {
   int32_t staged_threads;    /* threads of a staged block (three rows each); 0: the
                                 graph has none                                      */
   int32_t staged_rows;       /* rows of X the largest block stages                 */
-  int32_t staged_used;       /* the autotuner chose them for the products that can  */
+  int32_t staged_used;       /* the autotuner chose them, for the products that can
+                                use them and gain by it                              */
+  int32_t staged_last;       /* the handle's last product used them                  */
   int32_t lane_variant;      /* schedule of the products that cannot (spmm_variant
                                 where nothing is staged)                            */
   int32_t degree_slices;     /* F64 products use degree-ordered slices              */
@@ -271,7 +274,8 @@ int sphynx_get_plan_info(sphynx_handle g, sphynx_plan_info *info);
 
 /* Pin the short-row SpMM schedule of the handle: 0 = CSR staged in shared
  * memory, 1 = SELL-32, 2 = SELL-32 with shared-pattern slices (only when the
- * graph has such slices, see sphynx_graph_info), -1 = time them again and keep
+ * graph has such slices, see sphynx_graph_info; staged blocks wherever the
+ * product can use them), -1 = time them again and keep
  * the fastest (what sphynx_create does).  All give the same products up to
  * rounding order; 1 and 2 sum every row in the same order.
  * Errors: INVALID_ARG. */

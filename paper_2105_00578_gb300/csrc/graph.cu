@@ -877,13 +877,12 @@ void build_sell(sphynx_graph *g) {
 
 // Staged blocks, for graphs whose every slice is a shared-pattern slice and
 // whose rows average at least 16 entries: a staged row is then reused often
-// enough to pay for its copy.  Float products, us, staged against lane-per-row
-// kernel: 27-point meshes 80 x 75 x 70 17.2 / 28.9 and 128^3 73.7 / 121 (8
-// columns), 128^3 119 / 119 (12 columns), 210 / 406 (16 columns); the 5-point
-// mesh 1400^2 39.3 / 43.3, but 57.6 / 49.4 with 12 columns.  Blocks of 128
-// threads (384 rows); 64 where that leaves fewer than two blocks an SM (27-point
-// 48 x 40 x 44: 6.2 against 8.2 us).  256 threads measured the same at 128^3
-// (72.4) and 30.9 against 28.8 us at 101 x 97 x 89.
+// enough to pay for its copy (the 5-point mesh 1400^2 took 39.3 us against 43.3
+// with 8 float columns, but 57.6 against 49.4 with 12).  Which products use them
+// follows from their width and type and from rho, see blocks_pay in spmm.cu.
+// Blocks of 128 threads (384 rows); 64 where that leaves fewer than two blocks an
+// SM (27-point 48 x 40 x 44: 6.2 against 8.2 us).  256 threads measured the same
+// at 128^3 (72.4) and 30.9 against 28.8 us at 101 x 97 x 89.
 void build_blocks(sphynx_graph *g) {
   SpmmPlan &p = g->plan;
   p.blk_threads = 0;
@@ -1233,6 +1232,7 @@ int sphynx_get_plan_info(sphynx_handle g, sphynx_plan_info *info) {
     info->staged_rows = p.blk_threads ? p.blk_staged_rows : 0;
     info->staged_used = p.blk_threads && p.tuned_staged ? 1 : 0;
     info->lane_variant = p.lane_variant;
+    info->staged_last = p.stage_now ? 1 : 0;
     info->degree_slices = p.deg_row.p ? 1 : 0;
     info->tuned_us_staged = p.tuned_us_staged;
     for (int k = 0; k < kSellLsCount; ++k) info->tuned_us_stride[k] = p.tuned_ls_us[k];

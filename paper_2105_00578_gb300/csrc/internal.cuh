@@ -130,7 +130,7 @@ __device__ __forceinline__ int64_t sell_slot_row(const uint16_t *order, int64_t 
 
 struct SpmmTuning {
   int variant;                       // the fastest lane-per-row schedule
-  bool staged;                       // staged blocks are faster still
+  bool staged;                       // staged blocks are as fast or faster
   float us[kSpmmVariants];           // measured time of each schedule (1e30: not available)
   float us_staged;                   // and of the staged blocks
 };

@@ -106,6 +106,48 @@ bool blocks_take(const sphynx_graph *g, const SpmmArgs &a) {
          static_cast<size_t>(g->plan.blk_staged_rows) * a.bp * dt_size(a.tin) <= kBlkSmemMax;
 }
 
+// Do the staged blocks pay for this product?  A block stages rho rows of X per
+// row of Y: 3 at least on a 27-point mesh (one range a plane), 5 at 128 x 128 x nz,
+// 6.4 at lines of 220, and 9 from 384 on, where every line is a range of its own.
+// Their price is that copy, fewer resident warps the wider the rows are (float
+// rows of 12 leave one block an SM above rho = 6), and an accumulator Y that a
+// thread reads and writes three rows at a time where the lane-per-row kernel's
+// rows are adjacent.  So the line depends on the type, the width, what the
+// product does with Y, rho, and the blocks an SM has to run one after another.
+// Staged over lane-per-row time, measured on 19 meshes of 8,000 to 2,097,152 rows,
+// rho 3.5 to 9.1 (plain: a product, or a step that leaves Y alone; first: Y is
+// written; adds: Y is read and written); columns 4 | 8 | 12 | 16:
+//   float, plain    0.64-1.00, 1.04 at 9.1 | 0.45-1.00 | 0.76-1.01 up to 6, 1.33-1.55 above | 0.31-1.00
+//   float, first    0.71-1.16              | 0.50-1.02 | 0.81-1.11, 1.4-1.6               | 0.38-1.00
+//   float, adds     0.86-1.32              | 0.61-1.31 | 0.95-1.22, 1.7-1.9               | 0.45-1.00
+//   bfloat16, plain 0.79-1.46              | 0.74-1.24 | 0.79-1.43                        | 0.61-1.23
+//   bfloat16, first 0.78-1.33              | 0.88-1.32 | 0.91-1.52                        | 0.78-1.30
+//   bfloat16, adds  0.83-1.33              | 1.03-1.49 | 1.05-1.63                        | 0.85-1.33
+// (the high ends at few rows or rho above 7); within these lines 0.31 to 1.03.
+struct StageRule {
+  float blocks;   // least rows, in blocks of 3 kBlkThreads rows an SM
+  float rho;      // largest rho
+};
+constexpr float kNever = 1e30f, kAnyRho = 1e30f;
+constexpr StageRule kStageRules[2][4][3] = {   // [float, bfloat16][columns / 4 - 1][plain, first, adds]
+    {{{0, 8.5f}, {6, 7.5f}, {6, 6.5f}},
+     {{0, kAnyRho}, {0, kAnyRho}, {1, 8.5f}},
+     {{0, 6.f}, {kNever, 0}, {kNever, 0}},
+     {{0, kAnyRho}, {0, kAnyRho}, {0, kAnyRho}}},
+    {{{4, 8.5f}, {6, 8.5f}, {6, 8.5f}},
+     {{4, 7.2f}, {6, 6.f}, {kNever, 0}},
+     {{4, 7.f}, {kNever, 0}, {kNever, 0}},
+     {{1, kAnyRho}, {1, 6.f}, {kNever, 0}}}};
+
+bool blocks_pay(const sphynx_graph *g, const SpmmArgs &a) {
+  const int role = a.mode == 0 || a.yterms == 0 ? 0 : (a.first ? 1 : 2);
+  const StageRule &r = kStageRules[a.tin == DT::BF16][a.bp / 4 - 1][role];
+  const SpmmPlan &p = g->plan;
+  const float block = 3.f * kBlkThreads * kSmCount;
+  return static_cast<float>(g->n) >= r.blocks * block &&
+         static_cast<float>(p.blk_staged_rows) <= r.rho * 3.f * static_cast<float>(p.blk_threads);
+}
+
 struct TuneEvents {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   TuneEvents() {
@@ -163,8 +205,10 @@ SpmmTuning spmm_tune(sphynx_graph *g, const SpmmArgs &a) {
   g->plan.stage_now = false;
   for (int v = 1; v < nv; ++v)
     if (t.us[v] < t.us[t.variant]) t.variant = v;
-  // blocks too wide for this product may still serve narrower ones: with the layout's own result
-  t.staged = blocks ? t.us_staged < t.us[t.variant] : g->plan.blk_threads > 0 && t.variant == kSellPattern;
+  // A tie (small meshes, launches of a few us) goes to the blocks: wider products gain
+  // by them.  Blocks too wide for this product may still serve narrower ones: with
+  // the layout's own result.
+  t.staged = blocks ? t.us_staged <= 1.05f * t.us[t.variant] : g->plan.blk_threads > 0 && t.variant == kSellPattern;
   return t;
 }
 
@@ -249,7 +293,7 @@ void spmm(sphynx_graph *g, const SpmmArgs &a) {
   // wherever those exist (300,000-vertex geometric graph, 4 columns, a chain
   // step: 59.5 us in the CSR schedule, 39.2 in these).
   SpmmPlan &p = g->plan;
-  p.stage_now = (p.forced >= 0 ? p.forced == kSellPattern : p.tuned_staged) && blocks_take(g, a);
+  p.stage_now = blocks_take(g, a) && (p.forced >= 0 ? p.forced == kSellPattern : p.tuned_staged && blocks_pay(g, a));
   p.variant = p.forced >= 0 ? p.forced
               : p.stage_now ? static_cast<int>(kSellPattern)
               : a.tin == DT::F64 && p.deg_row.p ? static_cast<int>(kSell32) : p.lane_variant;
