@@ -191,8 +191,8 @@ typedef struct {
                                 Where 2 means staged blocks, F64 and normalized
                                 products and the widths and steps that gain nothing
                                 from them take the fastest of the other kernels
-                                (sphynx_plan_info), and F64 products use degree-
-                                ordered SELL-32 slices where the graph has them   */
+                                (sphynx_plan_info); F64 products use degree-ordered
+                                SELL-32 slices where the graph has them and they pay */
   float tuned_us_csr;        /* the two schedules' times for that product (us)    */
   float tuned_us_sell;
   int64_t sell_slices;       /* SELL-32 slices (32 rows each)                      */
@@ -230,7 +230,8 @@ typedef struct {
   int32_t staged_last;       /* the handle's last product used them                  */
   int32_t lane_variant;      /* schedule of the products that cannot (spmm_variant
                                 where nothing is staged)                            */
-  int32_t degree_slices;     /* F64 products use degree-ordered slices              */
+  int32_t degree_slices;     /* F64 products have degree-ordered slices             */
+  int32_t degree_last;       /* the handle's last product used them                 */
   float tuned_us_staged;     /* staged float 8-column product (us); 0: not timed    */
   float tuned_us_stride[5];  /* the lane-per-row SELL kernel at slice strides 1, 2,
                                 4, 8, 16; 0: not timed                              */

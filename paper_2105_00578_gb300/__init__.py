@@ -79,7 +79,8 @@ class GraphInfo(C.Structure):
 
 class PlanInfo(C.Structure):
     _fields_ = [("staged_threads", C.c_int32), ("staged_rows", C.c_int32), ("staged_used", C.c_int32),
-                ("staged_last", C.c_int32), ("lane_variant", C.c_int32), ("degree_slices", C.c_int32), ("tuned_us_staged", C.c_float),
+                ("staged_last", C.c_int32), ("lane_variant", C.c_int32), ("degree_slices", C.c_int32),
+                ("degree_last", C.c_int32), ("tuned_us_staged", C.c_float),
                 ("tuned_us_stride", C.c_float * 5)]
 
 

@@ -790,12 +790,14 @@ SliceLayout fill_slices(sphynx_graph *g, const SliceStats &st, const uint16_t *o
 // runs to the longest row of its slice, and a geometric graph's longest of 32
 // rows has nearly twice the mean.  300,000-vertex geometric graph, 4 columns:
 // chain step 61 -> 39 us.  Float products of that graph take 21 us in natural
-// order and 24 in this one.  Only for graphs of short rows without
-// shared-pattern slices (meshes: their rows are equally long already).
+// order and 24 in this one.  Only for graphs of short rows, and not where most
+// slices have a shared pattern (meshes: their rows are equally long already; a
+// geometric graph's ragged last slice of a few rows is often one by chance).
+// Which graphs and products they pay for: degrees_pay in spmm.cu.
 void build_degree_slices(sphynx_graph *g, int64_t natural_padded) {
   SpmmPlan &p = g->plan;
   p.deg_row.release();
-  if (p.pat_slices > 0 || g->max_degree > kShortDeg || g->n <= 32) return;
+  if (2 * p.pat_slices > (g->n + 31) / 32 || g->max_degree > kShortDeg || g->n < kDegMinRows) return;
   const int64_t n = g->n;
   p.deg_row.alloc(static_cast<size_t>(n) * sizeof(uint16_t));
   p.deg_deg.alloc(static_cast<size_t>(n));
@@ -1234,6 +1236,7 @@ int sphynx_get_plan_info(sphynx_handle g, sphynx_plan_info *info) {
     info->lane_variant = p.lane_variant;
     info->staged_last = p.stage_now ? 1 : 0;
     info->degree_slices = p.deg_row.p ? 1 : 0;
+    info->degree_last = p.degree_now && p.variant == kSell32 ? 1 : 0;
     info->tuned_us_staged = p.tuned_us_staged;
     for (int k = 0; k < kSellLsCount; ++k) info->tuned_us_stride[k] = p.tuned_ls_us[k];
     return SPHYNX_OK;

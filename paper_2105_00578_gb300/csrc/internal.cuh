@@ -121,6 +121,7 @@ constexpr int64_t kPatternTag = int64_t{1} << 62;
 
 constexpr int kBlkThreads = 128;                 // threads of a staged block, or half of them (three rows each)
 constexpr size_t kBlkSmemMax = 200 * 1024;       // shared memory a staged block may take
+constexpr int64_t kDegMinRows = 9 * 32 * kSmCount;   // degree-ordered slices: least rows, nine slices an SM
 constexpr int kSellLsCount = 5;      // slice strides 1, 2, 4, 8, 16 the autotuner times
 
 // the row of a SELL-32 slot (order: SpmmPlan::deg_row, NULL for natural order)
@@ -142,6 +143,7 @@ struct SpmmPlan {
   bool tuned_staged = false;         // blocks won, which the products that cannot use them
   int lane_variant = kCsrStaged;     // replace by the fastest lane-per-row schedule
   bool stage_now = false;            // the launch being issued uses the staged blocks
+  bool degree_now = false;           // or the degree-ordered slices
   float tuned_us[kSpmmVariants] = {0.f, 0.f, 0.f};   // its timings of the lane-per-row schedules
   float tuned_us_staged = 0.f;       // and of the staged blocks
   int sell_ls = 0;                   // SELL blocks: warps take slices 2^sell_ls apart

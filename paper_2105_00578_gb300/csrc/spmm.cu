@@ -148,6 +148,19 @@ bool blocks_pay(const sphynx_graph *g, const SpmmArgs &a) {
          static_cast<float>(p.blk_staged_rows) <= r.rho * 3.f * static_cast<float>(p.blk_threads);
 }
 
+// Double products in degree-ordered slices: their time over the better of the CSR
+// and the natural SELL schedule, geometric graphs, 1 to 16 columns.  Below nine
+// slices an SM (kDegMinRows: none are built) a warp's three dependent loads of
+// order, degree and column are not hidden: 1.00 to 1.32 at 500 to 32,000 rows, with
+// single cases down to 0.84.  From there on 0.55 to 1.01, but for normalized
+// products without weights, whose D^-1/2_j are gathered in the scattered order as
+// well: up to 1.24 below 13 slices an SM, and 1.08 to 1.27 for a single column at
+// any size.
+bool degrees_pay(const sphynx_graph *g, const SpmmArgs &a) {
+  if (a.tin != DT::F64 || !g->plan.deg_row.p) return false;
+  return a.lap != SPHYNX_NORMALIZED || g->weighted || (a.bp > 1 && g->n >= 13 * 32 * kSmCount);
+}
+
 struct TuneEvents {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   TuneEvents() {
@@ -289,14 +302,13 @@ void spmm(sphynx_graph *g, const SpmmArgs &a) {
   }
 
   // schedule: forced, or the one the autotuner chose for this graph at create
-  // from a float product.  Double products take the degree-ordered slices
-  // wherever those exist (300,000-vertex geometric graph, 4 columns, a chain
-  // step: 59.5 us in the CSR schedule, 39.2 in these).
+  // from a float product
   SpmmPlan &p = g->plan;
   p.stage_now = blocks_take(g, a) && (p.forced >= 0 ? p.forced == kSellPattern : p.tuned_staged && blocks_pay(g, a));
   p.variant = p.forced >= 0 ? p.forced
               : p.stage_now ? static_cast<int>(kSellPattern)
-              : a.tin == DT::F64 && p.deg_row.p ? static_cast<int>(kSell32) : p.lane_variant;
+              : degrees_pay(g, a) ? static_cast<int>(kSell32) : p.lane_variant;
+  p.degree_now = a.tin == DT::F64 && p.deg_row.p && (p.forced >= 0 || degrees_pay(g, a));
 
   // algorithmic bytes: the graph in the layout the schedule reads (CSR row
   // pointers and indices, or the SELL-32 slices plus the long rows' CSR

@@ -1326,7 +1326,7 @@ void spmm_launch_t(sphynx_graph *g, const SpmmDev &a) {
       const int ls = p.sell_ls;
       const unsigned gs = a.act_blocks ? static_cast<unsigned>(kListGrid)
                                        : static_cast<unsigned>(((warps + (int64_t{4} << ls) - 1) >> (ls + 2)) << ls);
-      const bool by_deg = std::is_same<TI, double>::value && p.variant == kSell32 && p.deg_row.p;
+      const bool by_deg = std::is_same<TI, double>::value && p.variant == kSell32 && p.degree_now;
       const int16_t *sc = (by_deg ? p.deg_col : p.sell_col).as<int16_t>();
       const float *swp = a.coef_sell ? a.coef_sell : (by_deg ? p.deg_w : p.sell_w).as<float>();
       const int64_t *sp = (by_deg ? p.deg_ptr : p.sell_ptr).as<int64_t>();
