@@ -45,6 +45,7 @@ int sphynx_gram(int32_t dtype, const void *const *s_blocks, const void *const *l
     launch_gram_reduce(st, part, nblk, ld, pg, ga, gb, nullptr);
     std::vector<double> out(2 * mm);   // both matrices in one copy
     SPX_CUDA(cudaMemcpyAsync(out.data(), ga, 2 * mm * 8, cudaMemcpyDeviceToHost, st));
+    scratch.release();
     SPX_CUDA(cudaStreamSynchronize(st));
     memcpy(ga_out, out.data(), mm * 8);
     memcpy(gb_out, out.data() + mm, mm * 8);
@@ -74,6 +75,7 @@ int sphynx_rayleigh_ritz(const double *ga, const double *gb, const int32_t *acti
     launch_rayleigh_ritz(st, dga, dga + mm, m, nev, nev, u_work, nullptr, dy, nullptr, DT::F64,
                          reinterpret_cast<int *>(dga + 2 * mm), dth, reinterpret_cast<int *>(dth + nev), 0);
     SPX_CUDA(cudaMemcpyAsync(out.data(), dy, outn * 8, cudaMemcpyDeviceToHost, st));
+    scratch.release();
     SPX_CUDA(cudaStreamSynchronize(st));
     int sv = 0;
     memcpy(&sv, out.data() + my + nev, 4);

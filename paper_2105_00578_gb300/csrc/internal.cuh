@@ -79,7 +79,13 @@ struct Scratch {
   void *p = nullptr;
   cudaStream_t st;
   Scratch(size_t bytes, cudaStream_t stream);   // throws OOM
-  ~Scratch() { if (p) cudaFreeAsync(p, st); }
+  ~Scratch() { release(); }
+  // The pool gives up what it holds beyond kScratchKeep at a synchronisation that
+  // follows the release, so that calls which synchronise release first.
+  void release() {
+    if (p) cudaFreeAsync(p, st);
+    p = nullptr;
+  }
   Scratch(const Scratch &) = delete;
   Scratch &operator=(const Scratch &) = delete;
 };
