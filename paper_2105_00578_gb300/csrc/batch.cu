@@ -1407,8 +1407,8 @@ void batch_partition(sphynx_graph *g, int K, const sphynx_options *o, int32_t *d
   SPX_LAUNCHED();
   // multi-jagged over all graphs at once: graph q owns parts [q K, (q + 1) K)
   const int ktot = count * K;
-  const size_t mj_bytes = mj_scratch_bytes(n, ktot, count, dt);
-  void *mjs = g->workspace("mj", mj_bytes, false);
+  size_t mj_bytes = 0;
+  void *mjs = mj_workspace(g, n, ktot, count, dt, &mj_bytes);
   const int64_t *vw_caller = orig && B.vw_orig.p ? B.vw_orig.as<int64_t>() : g->vw;
   run_mj_scratch(st, dt, coords, d - 1, d - 1, n, vw_caller, ktot, dpart, &g->ctr, mjs, mj_bytes, B.h_gptr.data(), count);
   // metrics per graph

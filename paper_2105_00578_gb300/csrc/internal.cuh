@@ -548,6 +548,8 @@ void run_mj(cudaStream_t st, DT dt, const void *coords, int ldc, int dims, int64
 // (host offsets) and parts [g K/count, (g+1) K/count): the first level has one
 // section per graph and every later level splits within them.
 size_t mj_scratch_bytes(int64_t n, int K, int count, DT dt);
+// a handle's workspace of that size, or of the least that serves if memory is short
+void *mj_workspace(sphynx_graph *g, int64_t n, int K, int count, DT dt, size_t *bytes);
 void run_mj_scratch(cudaStream_t st, DT dt, const void *coords, int ldc, int dims, int64_t n,
                     const int64_t *vw, int K, int32_t *part, Counters *ctr, void *scratch, size_t scratch_bytes,
                     const int64_t *h_gptr, int count);

@@ -711,8 +711,8 @@ int sphynx_partition(sphynx_handle g, int32_t K, const sphynx_options *opt, int3
     void *coords = g->workspace("coords", static_cast<size_t>(g->n) * (d - 1) * es + 16, false);
     double *sc = static_cast<double *>(g->workspace("signs", static_cast<size_t>(vec_grid(g->n)) * d * 3 * 8 + 16 * 8, false));
     launch_signs_coords(st, r.dt, r.x, g->n, r.ld, d, coords, sc);
-    const size_t mj_bytes = mj_scratch_bytes(g->n, K, 1, r.dt);
-    void *mjs = g->workspace("mj", mj_bytes, false);
+    size_t mj_bytes = 0;
+    void *mjs = mj_workspace(g, g->n, K, 1, r.dt, &mj_bytes);
     run_mj_scratch(st, r.dt, coords, d - 1, d - 1, g->n, g->vw, K, dpart, &g->ctr, mjs, mj_bytes, nullptr, 1);   // multi-jagged partition
     g->ctr.launches += 3;
     int refine_moves = 0;

@@ -32,6 +32,7 @@
 #include "internal.cuh"
 
 #include <cstring>
+#include <memory>
 #include <mutex>
 
 namespace sphynx {
@@ -501,6 +502,27 @@ MjPlan mj_plan(int64_t n, int K, int count, DT dt, size_t limit) {
 
 size_t mj_scratch_bytes(int64_t n, int K, int count, DT dt) { return mj_plan(n, K, count, dt, SIZE_MAX).bytes; }
 
+namespace {
+// alloc() of `bytes`; where the memory is short, of the least that serves
+template <class F> void or_least(size_t &bytes, size_t least, F alloc) {
+  try {
+    alloc();
+  } catch (const Error &e) {
+    if (e.code != SPHYNX_ERR_OOM || bytes <= least) throw;
+    clear_error();
+    bytes = least;
+    alloc();
+  }
+}
+}  // namespace
+
+void *mj_workspace(sphynx_graph *g, int64_t n, int K, int count, DT dt, size_t *bytes) {
+  void *p = nullptr;
+  *bytes = mj_scratch_bytes(n, K, count, dt);
+  or_least(*bytes, mj_least_bytes(n, K, count), [&] { p = g->workspace("mj", *bytes, false); });
+  return p;
+}
+
 void run_mj_scratch(cudaStream_t st, DT dt, const void *coords, int ldc, int dims, int64_t n, const int64_t *vw,
                     int K, int32_t *part, Counters *ctr, void *scratch, size_t scratch_bytes, const int64_t *h_gptr,
                     int count) {
@@ -697,9 +719,10 @@ void run_mj_scratch(cudaStream_t st, DT dt, const void *coords, int ldc, int dim
 
 void run_mj(cudaStream_t st, DT dt, const void *coords, int ldc, int dims, int64_t n, const int64_t *vw, int K,
             int32_t *part, Counters *ctr) {
-  const size_t bytes = mj_scratch_bytes(n, K, 1, dt);
-  Scratch scratch(bytes, st);
-  run_mj_scratch(st, dt, coords, ldc, dims, n, vw, K, part, ctr, scratch.p, bytes, nullptr, 1);
+  size_t bytes = mj_scratch_bytes(n, K, 1, dt);
+  std::unique_ptr<Scratch> scratch;
+  or_least(bytes, mj_least_bytes(n, K, 1), [&] { scratch.reset(new Scratch(bytes, st)); });
+  run_mj_scratch(st, dt, coords, ldc, dims, n, vw, K, part, ctr, scratch->p, bytes, nullptr, 1);
 }
 
 }  // namespace sphynx
