@@ -813,6 +813,26 @@ void build_degree_slices(sphynx_graph *g, int64_t natural_padded) {
                              p.deg_w).narrow;
 }
 
+// The layouts that only make products faster: where the memory is short for one, or
+// for what create needs after it, a handle goes without.
+void drop_extra_layouts(sphynx_graph *g) {
+  SpmmPlan &p = g->plan;
+  for (DevBuf *b : {&p.deg_row, &p.deg_ptr, &p.deg_cptr, &p.deg_col, &p.deg_w, &p.deg_deg, &p.blk_desc, &p.blk_mask})
+    b->release();
+  p.blk_threads = 0;
+}
+
+template <class F> void or_without_extra_layouts(sphynx_graph *g, F build, bool again) {
+  try {
+    build();
+  } catch (const Error &e) {
+    if (e.code != SPHYNX_ERR_OOM || (again && !g->plan.deg_row.p && !g->plan.blk_threads)) throw;
+    clear_error();
+    drop_extra_layouts(g);
+    if (again) build();
+  }
+}
+
 void build_sell(sphynx_graph *g) {
   SpmmPlan &p = g->plan;
   const int64_t n = g->n, slices = (n + 31) / 32;
@@ -874,7 +894,7 @@ void build_sell(sphynx_graph *g) {
     SPX_LAUNCHED();
   }
   SPX_CUDA(cudaStreamSynchronize(g->stream));
-  build_degree_slices(g, st.padded());
+  or_without_extra_layouts(g, [&] { build_degree_slices(g, st.padded()); }, false);
 }
 
 // Staged blocks, for graphs whose every slice is a shared-pattern slice and
@@ -1173,8 +1193,8 @@ int sphynx_create(const int64_t *row_ptr, const int32_t *col, const float *edge_
     build_plan(g.get(), dev ? nullptr : row_ptr, kMedDeg);
     g->plan.prescale = g->max_degree * g->n > 10 * g->nnz;   // irregular: max degree above 10 x the mean
     build_sell(g.get());
-    build_blocks(g.get());
-    autotune_spmm(g.get(), dev ? nullptr : row_ptr);
+    or_without_extra_layouts(g.get(), [&] { build_blocks(g.get()); }, false);
+    or_without_extra_layouts(g.get(), [&] { autotune_spmm(g.get(), dev ? nullptr : row_ptr); }, true);
     *out = g.release();
     return SPHYNX_OK;
   });

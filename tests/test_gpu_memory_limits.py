@@ -40,3 +40,31 @@ def test_multijagged_without_room_for_its_keys():
         spx.sphynx_mj(spx.DT_F64, c, 2, 2, n, None, K, got)
         torch.cuda.synchronize()
     assert torch.equal(ref, got)
+
+
+def _least_create(torch, g, before):
+    """The least free memory (in steps of 8 MB) in which sphynx_create succeeds, and the plan it then has."""
+    import paper_2105_00578_gb300 as spx
+    for mb in range(64, 4096, 8):
+        before()
+        with only(torch, mb << 20):
+            try:
+                h = spx.sphynx_create(g.row_ptr, g.col)
+            except spx.SphynxError as e:
+                assert e.code == spx.ERR_OOM
+                continue
+            plan = spx.sphynx_get_plan_info(h)
+            spx.sphynx_destroy(h)
+            return mb, plan
+    raise AssertionError("never fits")
+
+
+def test_create_goes_without_the_layouts_that_only_add_speed():
+    import paper_2105_00578_gb300 as spx
+    torch = torch_mod()
+    for g, field in ((W.rgg(1_200_000, seed=2), "degree_slices"), (W.grid3d(128, 128, 90, 27), "staged_threads")):
+        h = spx.sphynx_create(g.row_ptr, g.col)     # modules loaded
+        assert spx.sphynx_get_plan_info(h)[field] > 0
+        spx.sphynx_destroy(h)
+        mb, plan = _least_create(torch, g, lambda: None)
+        assert plan[field] == 0, (mb, plan)
