@@ -279,10 +279,9 @@ k_eval_short(const int16_t *__restrict__ scol, const float *__restrict__ sw, con
     if (in && !ok) bad = 1;
     unsigned long long wv = ok ? (vw ? static_cast<unsigned long long>(vw[row]) : 1ull) : 0ull;
     const int32_t p0 = __shfl_sync(0xffffffffu, pi, 0);
-    if (__all_sync(0xffffffffu, !ok || pi == p0)) {
+    if (__all_sync(0xffffffffu, !ok || pi == p0)) {   // with lane 0 out of range: no lane is in range
       for (int off = 16; off > 0; off >>= 1) wv += __shfl_down_sync(0xffffffffu, wv, off);
       if (lane == 0 && ok) atomicAdd(&weights[pi], wv);
-      else if (lane == 0 && wv) bad = 1;
     } else if (ok) {
       atomicAdd(&weights[pi], wv);
     }
