@@ -382,8 +382,8 @@ int sphynx_amg_level(sphynx_handle g, int32_t level, sphynx_amg_level_info *info
  * Accumulation: products in the input type, short sums in the input type,
  * then a (hi, lo) float pair (float input) or double, per-CTA partials in
  * double added in a fixed order.
- * Scratch: taken from a stream-ordered memory pool of the library on `stream`;
- * at most 64 MB stay in the pool between calls. */
+ * Scratch: taken from a stream-ordered memory pool of the library on `stream`,
+ * which holds at most 64 MB when the call returns. */
 int sphynx_gram(int32_t dtype, const void *const *s_blocks, const void *const *ls_blocks,
                 int32_t nblk, int32_t ld, int64_t n, const double *bdiag, double *ga_out,
                 double *gb_out, void *stream);
@@ -414,7 +414,8 @@ int sphynx_eigensolve(sphynx_handle g, const sphynx_options *opt, int32_t nev, c
  * ceil(k/2) | floor(k/2) along dimension (level mod dims) at the prefix of
  * the (coordinate, vertex id) order minimising |k W_left - ceil(k/2) W|,
  * ties to the shorter prefix (-0 == +0; NaN is INVALID_ARG).
- * part_out: device int32[n].  Scratch is allocated per call.  Bit-exact. */
+ * part_out: device int32[n].  Scratch is taken per call from the library's
+ * memory pool (less of it where memory is short).  Bit-exact. */
 int sphynx_mj(int32_t dtype, const void *coords, int32_t ldc, int32_t dims, int64_t n,
               const int64_t *vtx_w, int32_t K, int32_t *part_out, void *stream);
 
@@ -431,8 +432,8 @@ int sphynx_mj(int32_t dtype, const void *coords, int32_t ldc, int32_t dims, int6
  * call on a device looks up the array's device address
  * (cudaGetSymbolAddress) and should therefore come before any stream
  * capture.  Like sphynx_mj, every call reads two values back to the host (a
- * NaN / vertex-weight flag and the total vertex weight), so it synchronises
- * `stream` twice, and it uploads its section tables from pageable host
+ * NaN / vertex-weight flag and the total vertex weight, in one copy), so it
+ * synchronises `stream` once, and it uploads its section tables from pageable host
  * memory.  All calls share the one array and each call clears what it needs
  * cleared: calls whose GPU work overlaps (different streams, or concurrent
  * host threads) race and must be serialised by the caller. */

@@ -913,8 +913,10 @@ k_spmm_sell(const LapView L, const SpmmDev a, const int16_t *__restrict__ scol, 
 // 3 L entries.  The lane-per-row kernel is bound by the L1 data pipe (float
 // rows: 16 wavefronts an entry of 32 rows) and, in bfloat16, by issue (29
 // instructions an entry); this one has a third of both and is bound by the
-// latency of a block's copies.  128^3 27-point mesh: float product 122 -> 74 us,
-// bfloat16 chain step 57 -> 53 us.
+// latency of a block's copies (float; the bfloat16 one has no counters).  128^3
+// 27-point mesh: float product 122 -> 73 us, bfloat16 step that leaves Y alone
+// 51.5 -> 39 us.  A bfloat16 step that adds to Y takes 64 against 58 us: blocks_pay
+// in spmm.cu says which products run here.
 // Three rows a thread, not two or four: an odd stride keeps the 16-byte loads
 // of a quarter warp in different banks (two-chunk rows alternate which half
 // they load first).  Every row adds its entries one by one in ascending column
@@ -954,7 +956,8 @@ template <typename TI, int BP> struct StagedRow {
 
 // sums of staged rows: packed float pairs, or floats that take bfloat16 values
 // by the mixed-precision multiply-add (exact widening, full rate; unpacking to
-// packed pairs first took 59 instead of 53 us a chain step at 128^3)
+// packed pairs first took 59 instead of 53 us a step at 128^3, both kinds of step
+// averaged)
 template <typename TI, int BP> struct StagedAcc;
 template <int BP> struct StagedAcc<float, BP> {
   using S = StagedRow<float, BP>;
